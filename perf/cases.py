@@ -15,8 +15,8 @@ The data follow the library's synthetic workloads: a Gaussian mixture on the
 unit sphere, queries that are corpus points with noise, Zipf-sized tenants in
 shuffled order.  Corpora are drawn in the rotated basis (the mixture's
 distribution does not depend on the basis) and quantised here with torch, so
-that the codes a search reads do not depend on the encoder.  Queries go
-through a created stream, as a serving loop does.
+that the codes a search reads do not depend on the encoder.  All
+passes go through one created stream, as in a serving loop.
 """
 import functools
 import math
@@ -85,6 +85,12 @@ def _codebook(d, bits):
     return c, t
 
 
+@functools.lru_cache(maxsize=1)
+def _stream():
+    """The serving loop's stream: one for all states, so that passes follow one another."""
+    return torch.cuda.Stream()
+
+
 def _generator(seed):
     g = torch.Generator(device="cuda")
     g.manual_seed(seed)
@@ -151,7 +157,7 @@ def prepare(case, seed):
     R = _rotation(d, g)
     c, t = (torch.from_numpy(v).cuda() for v in _codebook(d, bits))
     calib = _calibration(d, g) if case["tqplus"] else None
-    s = {"case": case, "R": R, "c": c, "t": t, "calib": calib, "stream": torch.cuda.Stream()}
+    s = {"case": case, "R": R, "c": c, "t": t, "calib": calib, "stream": _stream()}
     if case["kind"] == "encode":
         s["X"] = torch.empty(n, d, device="cuda")
         for a, y in _mixture(n, d, g):
