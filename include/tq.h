@@ -269,9 +269,12 @@ tq_status tq_search_workspace(int64_t nq, int64_t n, int d, int bits, int k,
  *   out_scores     device out [nq*k] float32, -INFINITY where out_ids is -1
  *   workspace      device scratch of ws_bytes >= tq_search_workspace(...)
  * Kernels (TQ_PATH_AUTO): batches of 16 or more queries over 2-, 4- or 8-bit
- * codes with d a multiple of 64 and k <= 64 run the tensor-core scan (fp16
- * products, float32 accumulation), filtered or not; the rest run the lookup
- * scan (float32 sums).
+ * codes with d a multiple of 64 and k <= 64 run a tensor-core scan (fp16
+ * products, float32 accumulation), filtered or not; the rest give the lookup
+ * scan's results (float32 sums).  Unfiltered batches below 16 over 4-bit codes
+ * (d a multiple of 256, k <= 32, enough rows) get them from a tensor-core scan
+ * that bounds every score and float32 scores of the candidates the bounds
+ * leave, bit for bit what the lookup scan returns.
  */
 tq_status tq_search(const float* Q, int64_t nq, int d, const float* R,
                     const float* centroids, int bits, const uint8_t* codes,

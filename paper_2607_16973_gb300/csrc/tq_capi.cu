@@ -30,14 +30,15 @@ constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct SearchPlan {
-  int grid_lut = 1, grid_mma = 0, grid_fold = 0;
-  size_t off_status = 0, off_cnt = 0, off_bias = 0, off_rot = 0, off_part = 0, off_allow = 0, off_mask = 0,
+  int grid_lut = 1, grid_mma = 0, grid_fold = 0, grid_tm = 0;
+  size_t off_status = 0, off_cnt = 0, off_bias = 0, off_gate = 0, off_lows = 0, off_rot = 0, off_part = 0, off_allow = 0, off_mask = 0,
          off_qpack = 0, off_cs = 0, off_ci = 0, total = 0;
   bool rot_tc = false;  // the query rotation runs on the tensor cores
 };
 
 // Workspace layout (both scan paths): status word | merge counters (one per
-// query) | TQ+ query terms (one per query) | rotated queries | partial
+// query, and the small-batch scan's thresholds and force word) | its gates (one per
+// query) and list bounds (two per query and CTA) | TQ+ query terms (one per query) | rotated queries | partial
 // rotations (tensor-core rotation) | allow bitmaps | block masks | fp16 query
 // tiles (tensor-core scan) | candidate scores | ids.
 SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_filter* filter) {
@@ -46,12 +47,19 @@ SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_f
   const bool mma = mma_supported(bits, d, k);
   p.grid_mma = mma ? scan_mma_grid_x(nq, n, k, bits) : 0;
   p.grid_fold = fold_supported(bits, d, k, n) ? scan_fold_grid_x(nq, n) : 0;
-  const int per_query = std::max(std::max(p.grid_lut, p.grid_mma), p.grid_fold) * k;
+  const bool tm = scan_tm_supported(nq, n, d, bits, k, true), tm16 = scan_tm_supported(nq, n, d, bits, k, false);
+  p.grid_tm = tm || tm16 ? scan_tm_grid_x(n) : 0;
+  const int per_query = std::max(std::max(std::max(p.grid_lut, p.grid_mma), p.grid_fold) * k,
+                                 p.grid_tm * scan_tm_list(k, tm));
   size_t off = 0;
   p.off_status = off;
   off = align_up(off + sizeof(int));
   p.off_cnt = off;
-  off = align_up(off + (size_t)nq * sizeof(int));
+  off = align_up(off + ((size_t)2 * nq + 1) * sizeof(int));
+  p.off_gate = off;
+  if (tm) off = align_up(off + (size_t)nq * sizeof(int));
+  p.off_lows = off;
+  if (tm) off = align_up(off + (size_t)2 * nq * p.grid_tm * sizeof(float));
   p.off_bias = off;
   off = align_up(off + (size_t)nq * sizeof(float));
   p.off_rot = off;
@@ -432,6 +440,10 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
   // AUTO keeps the byte-pair scan: on GB300 it is the faster of the two (218
   // against 228 us per query at 999,000 x 1536)
   const bool use_fold = !use_mma && can_fold && path == TQ_PATH_LUT_FOLD;
+  // AUTO: the small-batch tensor-core scan, exact (bounds, then float32
+  // scores) for unfiltered batches the lookup scan would take, fp16 above
+  const bool tm_bound = path == TQ_PATH_AUTO && !use_mma && !filter && tq::scan_tm_supported(nq, n, d, bits, k, true);
+  const bool use_tm = tm_bound || (path == TQ_PATH_AUTO && use_mma && tq::scan_tm_supported(nq, n, d, bits, k, false));
   const tq::SearchPlan p = tq::plan_search(nq, n, d, bits, k, filter);
   if (ws_bytes < p.total)
     return fail(TQ_EINVAL, "tq_search: workspace of %zu bytes, %zu needed", ws_bytes, p.total);
@@ -445,12 +457,33 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
   float* cs = reinterpret_cast<float*>(ws + p.off_cs);
   int32_t* ci = reinterpret_cast<int32_t*>(ws + p.off_ci);
   float* bias = cal_mu ? reinterpret_cast<float*>(ws + p.off_bias) : nullptr;
-  // the rotation also clears the status word and zeroes the merge counters
+  uint32_t* gth = reinterpret_cast<uint32_t*>(counters + nq);
+  int* force = counters + 2 * nq;
+  // the rotation also clears the status word and zeroes the counters, thresholds and the force word
   cudaError_t e = p.rot_tc ? tq::launch_rotate_tc(Q, nq, d, R, qrot, reinterpret_cast<float*>(ws + p.off_part),
-                                                  status, counters, nq, s)
-                           : tq::launch_rotate(Q, nq, d, R, qrot, status, counters, nq, s);
+                                                  status, counters, 2 * nq + 1, s)
+                           : tq::launch_rotate(Q, nq, d, R, qrot, status, counters, 2 * nq + 1, s);
   if (e == cudaSuccess && cal_mu) e = tq::launch_calib_query(qrot, nq, d, cal_mu, cal_a, bias, s);
-  if (use_mma) {
+  if (use_tm) {
+    float* lows = reinterpret_cast<float*>(ws + p.off_lows);
+    int* gate = reinterpret_cast<int*>(ws + p.off_gate);
+    if (e == cudaSuccess && filter) e = tq::launch_allow_bits(filter->f, allow_off, allow_tenants, nq, allow, s);
+    if (e == cudaSuccess)
+      e = tq::launch_scan_tm(qrot, nq, d, centroids, codes, scale, n, deleted, filter ? filter->f.dense : nullptr,
+                             allow, filter ? filter->f.words : 0, bias, k, tm_bound, cs, ci, status, force, gth, lows, s,
+                             (cudaEvent_t)tq::profile_start(), (cudaEvent_t)tq::profile_stop());
+    if (tm_bound) {
+      if (e == cudaSuccess)
+        e = tq::launch_rescore(qrot, nq, d, centroids, codes, scale, n, k, cs, ci, lows, force, gate, ext_ids, out_ids,
+                               out_scores, bias, s);
+      if (e == cudaSuccess)
+        e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, deleted, nullptr, nullptr, nullptr,
+                                false, k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias,
+                                gate, s, nullptr, nullptr);
+    } else if (e == cudaSuccess) {
+      e = tq::launch_merge(cs, ci, nq, p.grid_tm * k, k, ext_ids, out_ids, out_scores, s);
+    }
+  } else if (use_mma) {
     if (e == cudaSuccess && filter) e = tq::launch_allow_bits(filter->f, allow_off, allow_tenants, nq, allow, s);
     if (e == cudaSuccess)
       e = tq::launch_scan_mma(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
@@ -470,8 +503,8 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
       e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
                               filter ? &filter->f : nullptr, allow, bmask,
                               path == TQ_PATH_LUT_FIXED && d >= tq::kFixMinD,
-                              k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias, s,
-                              (cudaEvent_t)tq::profile_start(), (cudaEvent_t)tq::profile_stop());
+                              k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias,
+                              nullptr, s, (cudaEvent_t)tq::profile_start(), (cudaEvent_t)tq::profile_stop());
   }
   if (e != cudaSuccess) return tq::cuda_fail("tq_search", e);
   return tq::ok();

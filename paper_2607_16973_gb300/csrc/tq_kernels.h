@@ -84,14 +84,15 @@ cudaError_t launch_filter_raw_ids(const FilterDev& f, uint32_t* raw, cudaStream_
 // last CTA of each query merges the CTA lists into out_ids/out_scores
 // (written as ext[row] with an id map); `counters` [nq] must be zero (the
 // query rotation zeroes them).  `bias` [nq] (nullable): a TQ+ search's
-// per-query term, added to each raw score before the per-vector scale.
+// per-query term, added to each raw score before the per-vector scale.  `gate`
+// [nq] (nullable; not for 3-bit codes): only queries with gate[q] != 0 are searched.
 int scan_lut_grid_x(int64_t nq, int64_t n, int k, int bits, int d);
 cudaError_t launch_scan_lut(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
                             const uint8_t* codes, const float* scale, int64_t n, const uint32_t* del,
                             const FilterDev* f, const uint32_t* allow_bits, const uint32_t* bmask, bool fix,
                             int k, int grid_x, float* cand_s, int32_t* cand_i, int* err, int* counters,
                             const uint64_t* ext, int64_t* out_ids, float* out_scores, const float* bias,
-                            cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1);
+                            const int* gate, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1);
 
 // The 4-bit lookup scan with the rotated query folded into per-byte-position
 // tables (k_scan_fold): bits 4, d >= 256 and a multiple of 32, k <= kFoldMaxK,
@@ -133,6 +134,28 @@ cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* c
                             const uint32_t* dense, const uint32_t* allow_bits, int words, const float* bias,
                             int k, int grid_x, void* qpack, float* cand_s, int32_t* cand_i, int* err, cudaStream_t s,
                             cudaEvent_t ev0, cudaEvent_t ev1);
+
+// Small-batch tensor-core scan of 4-bit codes (k_scan_tm).  With `bound` it is
+// the first half of an exact float32 search of at most 16 queries: every CTA
+// keeps the scan_tm_list(k, true) vectors whose upper score bounds are best,
+// and launch_rescore scores the candidates as the lookup scan does, writes the
+// results and sets gate[q] for the queries it could not settle (the lookup
+// scan then runs for those).  `gth` [nq]: thresholds the CTAs share; `force` is raised
+// for values the bounds do not cover (both zeroed by the query rotation); lows [2][nq][grid_x] are lower bounds of
+// each list's best and k-th best score.
+// Without it, fp16 scores of at most 32 queries: lists of k for launch_merge.
+bool scan_tm_supported(int64_t nq, int64_t n, int d, int bits, int k, bool bound);
+int scan_tm_list(int k, bool bound);
+int scan_tm_grid_x(int64_t n);
+cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* centroids, const uint8_t* codes,
+                           const float* scale, int64_t n, const uint32_t* del, const uint32_t* dense,
+                           const uint32_t* allow_bits, int words, const float* bias, int k, bool bound, float* cand_s,
+                           int32_t* cand_i, int* err, int* force, uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
+                           cudaEvent_t ev1);
+cudaError_t launch_rescore(const float* qrot, int64_t nq, int d, const float* centroids, const uint8_t* codes,
+                           const float* scale, int64_t n, int k, const float* cand_s, const int32_t* cand_i,
+                           const float* lows, const int* force, int* gate, const uint64_t* ext, int64_t* out_ids,
+                           float* out_scores, const float* bias, cudaStream_t s);
 
 int device_sm_count();
 cudaError_t set_max_dynamic_smem(const void* func, int bytes);

@@ -335,7 +335,11 @@ k_scan_stream(const float* __restrict__ qrot, int d, const float* __restrict__ c
               const uint32_t* __restrict__ allow_bits, int words, const uint32_t* __restrict__ bmask,
               int mask_words, int fblock, int k, int P, float* __restrict__ cand_s, int* __restrict__ cand_i,
               int* __restrict__ counters, const uint64_t* __restrict__ ext, int64_t* __restrict__ out_ids,
-              float* __restrict__ out_scores, const float* __restrict__ bias) {
+              float* __restrict__ out_scores, const float* __restrict__ bias, const int* __restrict__ gate) {
+  if (gate) {  // behind an exact tensor-core search: only the queries it could not settle
+    griddep_wait();
+    if (!__ldcg(gate + blockIdx.y)) return;
+  }
   constexpr int L = 1 << BITS;
   constexpr int CB = 2 * BITS;   // bytes of a 16-code chunk
   constexpr int V = 4;           // vectors per warp step; a CTA step covers 32
@@ -926,26 +930,8 @@ struct ScanArgs {
   float* out_scores;
   bool pdl;
   const float* bias;
+  const int* gate;
 };
-
-// Launches `kernel`, with programmatic stream serialization when `pdl` (the
-// kernel then overlaps the tail of the one before it and waits for it with
-// griddep_wait before reading its results).
-template <typename... Params, typename... Args>
-cudaError_t launch_maybe_pdl(bool pdl, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
-                             cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
 
 // Dynamic shared memory of the ring scan with `ns` slots per warp.
 constexpr size_t kRingSmemMax = 232448 - 2048;  // 227 KB less the static arrays
@@ -989,7 +975,7 @@ cudaError_t scan_typed(dim3 grid, size_t smem, cudaStream_t s, const ScanArgs& a
   return launch_maybe_pdl(a.pdl, k_scan_stream<BITS, S, FILT, FIX>, grid, dim3(SCAN_NT), smem, s, a.qrot, a.d,
                           a.centroids, a.codes, a.scale, a.n, a.del, a.dense, a.allow, a.words, a.bmask,
                           a.mask_words, a.fblock, a.k, a.P, a.cs, a.ci, a.counters, a.ext, a.out_ids, a.out_scores,
-                          a.bias);
+                          a.bias, a.gate);
 }
 
 template <int BITS, int S>
@@ -1037,7 +1023,7 @@ cudaError_t launch_scan_lut(const float* qrot, int64_t nq, int d, const float* c
                             const FilterDev* f, const uint32_t* allow_bits, const uint32_t* bmask, bool fix,
                             int k, int grid_x, float* cand_s, int32_t* cand_i, int* err, int* counters,
                             const uint64_t* ext, int64_t* out_ids, float* out_scores, const float* bias,
-                            cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1) {
+                            const int* gate, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1) {
   if (nq == 0) return cudaSuccess;
   const int S = (d + 511) / 512;
   const int P = next_pow2(SCAN_WARPS * k);
@@ -1049,7 +1035,7 @@ cudaError_t launch_scan_lut(const float* qrot, int64_t nq, int d, const float* c
              f ? f->block : 64, k, P, cand_s, cand_i, err, counters, ext, out_ids, out_scores,
              // overlap with the kernel before (not on the legacy default stream, and not
              // between profiling events, which would serialise the two anyway)
-             s != nullptr && ev0 == nullptr, bias};
+             s != nullptr && ev0 == nullptr, bias, gate};
   const bool filt = f != nullptr;
   cudaError_t e;
   if (ev0 && (e = cudaEventRecord(ev0, s)) != cudaSuccess) return e;

@@ -515,5 +515,24 @@ __device__ __forceinline__ void cta_lists_out(float* ls, int* li, int nw, int k,
   }
 }
 
+// Launches `kernel`, with programmatic stream serialization when `pdl` (the
+// kernel then overlaps the tail of the one before it and waits for it with
+// griddep_wait before reading its results).
+template <typename... Params, typename... Args>
+cudaError_t launch_maybe_pdl(bool pdl, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 }  // namespace
 }  // namespace tq

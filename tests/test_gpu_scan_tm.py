@@ -1,0 +1,172 @@
+"""The small-batch tensor-core scan of 4-bit codes (k_scan_tm).
+
+Below 16 queries it is the first half of an exact search: the scan keeps the
+vectors whose upper score bounds are best and k_rescore takes the lookup
+scan's float32 score of those, so ids and scores have to be the lookup scan's
+bit for bit, also where the bounds cannot settle a query (ties, duplicates) or
+do not cover the values (scales that are not finite) and the lookup scan runs
+after all.  From 16 to 32 queries its scores are fp16 products like the
+batched scan's and are checked against the oracle within its tolerance."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2607_16973_gb300 import synth
+from parity import TOL_LUT, TOL_MMA, check_topk
+from test_gpu_fold import _cb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tdev(cuda_lib):
+    import torch
+    dev = torch.device("cuda:0")
+    return torch, (lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev))
+
+
+def _data(n, d, nq, seed):
+    packed = synth.random_codes(n, d // 2, seed=seed)
+    scale = synth.random_scales(n, seed=seed)
+    R = O.rotation(d, 5).astype(np.float32)
+    Q = synth.gaussian_rows(nq, d, seed=seed)
+    Q /= np.linalg.norm(Q, axis=1, keepdims=True)
+    return packed, scale, R, Q
+
+
+def _search(tq, torch, path, *a, **kw):
+    tq.set_search_path(path)
+    try:
+        ids, sc = tq.search(*a, **kw)
+        torch.cuda.synchronize()
+    finally:
+        tq.set_search_path("auto")
+    return ids.cpu().numpy(), sc.cpu().numpy()
+
+
+# rows x d x queries of 2^24 and more (2^27 for k > 16) take the tensor-core scan
+@pytest.mark.parametrize("d,n,nq,k", [
+    (256, 65_537, 1, 1),       # one raw code tile per vector tile, one row past a tile
+    (256, 40_000, 15, 32),     # the largest batch and k
+    (512, 60_000, 9, 16),
+    (768, 25_001, 1, 10),
+    (1536, 11_000, 1, 10),     # fewer tiles than SMs
+    (1536, 70_001, 3, 7),      # four tiles per CTA
+    (2048, 20_000, 8, 5),      # the largest d
+])
+def test_exact_search_is_the_lookup_scan(cuda_lib, tdev, d, n, nq, k):
+    torch, T = tdev
+    tq = cuda_lib
+    packed, scale, R, Q = _data(n, d, nq, seed=d + nq)
+    scale[::97] *= -1.0
+    scale[5] = 0.0
+    c32, _ = _cb(d)
+    a = (T(Q), T(R), T(c32), 4, T(packed), T(scale), k)
+    ids, sc = _search(tq, torch, "auto", *a)
+    ids_l, sc_l = _search(tq, torch, "lut", *a)
+    assert np.array_equal(ids, ids_l) and np.array_equal(sc, sc_l)
+    ref = O.search(Q, R, c32, 4, packed, scale, k, d)
+    check_topk(ids, sc, ref.ids, ref.scores64, np.ones_like(ref.scores64, bool), k, TOL_LUT)
+
+
+def _all_equal(packed, scale, Q, c32):
+    packed[:], scale[:] = packed[7], scale[7]
+
+
+def _many_copies(packed, scale, Q, c32):  # more copies of a vector than a list holds, in one vector tile
+    packed[256:320], scale[256:320] = packed[7], scale[7]
+    Q[:] = Q[0]
+
+
+def _infinite_scale(packed, scale, Q, c32):
+    scale[100] = np.inf
+
+
+def _nan_scale(packed, scale, Q, c32):
+    scale[100] = np.nan
+
+
+def _zero_query(packed, scale, Q, c32):
+    Q[1] = 0.0
+
+
+def _huge_query(packed, scale, Q, c32):
+    Q *= np.float32(1e25)
+
+
+def _nan_query(packed, scale, Q, c32):
+    Q[1, 3] = np.nan
+
+
+def _wide_scales(packed, scale, Q, c32):
+    scale *= np.exp(synth.gaussian_rows(1, len(scale), seed=3)[0] * 4).astype(np.float32)
+
+
+def _infinite_centroid(packed, scale, Q, c32):
+    c32[15] = np.inf
+
+
+@pytest.mark.parametrize("change", [_all_equal, _many_copies, _infinite_scale, _nan_scale, _zero_query, _huge_query,
+                                    _nan_query, _wide_scales, _infinite_centroid])
+def test_exact_search_on_odd_values(cuda_lib, tdev, change):
+    torch, T = tdev
+    tq = cuda_lib
+    d, n, nq, k = 512, 20_000, 3, 10
+    packed, scale, R, Q = _data(n, d, nq, seed=11)
+    c32 = _cb(d)[0].copy()
+    change(packed, scale, Q, c32)
+    a = (T(Q), T(R), T(c32), 4, T(packed), T(scale), k)
+    ids, sc = _search(tq, torch, "auto", *a)
+    ids_l, sc_l = _search(tq, torch, "lut", *a)
+    assert np.array_equal(ids, ids_l) and np.array_equal(sc, sc_l, equal_nan=True)
+
+
+def test_exact_search_with_deleted_rows_and_calibration(cuda_lib, tdev):
+    torch, T = tdev
+    tq = cuda_lib
+    d, n, nq, k = 1024, 30_000, 5, 10
+    packed, scale, R, Q = _data(n, d, nq, seed=21)
+    c32, _ = _cb(d)
+    mu = (synth.gaussian_rows(1, d, seed=4)[0] * 0.01).astype(np.float32)
+    a_ = np.exp(synth.gaussian_rows(1, d, seed=5)[0] * 0.2).astype(np.float32)
+    m = tq.IdMap(n)
+    m.add(np.arange(n, dtype=np.uint64) + 10**9)
+    first, _ = _search(tq, torch, "lut", T(Q), T(R), T(c32), 4, T(packed), T(scale), k, idmap=m, calib=(T(mu), T(a_)))
+    m.remove(first[:, ::2].reshape(-1).view(np.uint64))  # half of what would be found
+    args = (T(Q), T(R), T(c32), 4, T(packed), T(scale), k)
+    got = _search(tq, torch, "auto", *args, idmap=m, calib=(T(mu), T(a_)))
+    want = _search(tq, torch, "lut", *args, idmap=m, calib=(T(mu), T(a_)))
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    assert not set(got[0].reshape(-1).tolist()) & set(first[:, ::2].reshape(-1).tolist())
+
+
+@pytest.mark.parametrize("d,n,nq,k", [
+    (256, 1, 16, 3),          # one row, k - 1 empty slots
+    (256, 129, 17, 1),        # one row past a tile, the wider query block
+    (1536, 3_000, 32, 32),    # the largest batch and k
+    (2048, 20_001, 20, 5),    # the largest d: two raw code stages
+])
+def test_fp16_batches(cuda_lib, tdev, d, n, nq, k):
+    torch, T = tdev
+    tq = cuda_lib
+    packed, scale, R, Q = _data(n, d, nq, seed=d + nq)
+    c32, _ = _cb(d)
+    ids, sc = _search(tq, torch, "auto", T(Q), T(R), T(c32), 4, T(packed), T(scale), k)
+    ref = O.search(Q, R, c32, 4, packed, scale, k, d)
+    check_topk(ids, sc, ref.ids, ref.scores64, np.ones_like(ref.scores64, bool), k, TOL_MMA)
+
+
+def test_fp16_batch_filtered(cuda_lib, tdev):
+    torch, T = tdev
+    tq = cuda_lib
+    d, n, nq, k = 512, 9_001, 24, 10
+    packed, scale, R, Q = _data(n, d, nq, seed=31)
+    c32, _ = _cb(d)
+    tenants, values = synth.zipf_tenants(n, 100)
+    off, ids_allowed = synth.allowlists(synth.query_sources(n, nq), tenants, values)
+    flt = tq.Filter(T(tenants.view(np.int32)), block=64)
+    ids, sc = _search(tq, torch, "auto", T(Q), T(R), T(c32), 4, T(packed), T(scale), k, filter=flt, allow_off=T(off),
+                      allow_tenants=T(ids_allowed.view(np.int32)))
+    allowed = np.stack([np.isin(tenants, ids_allowed[off[i]:off[i + 1]]) for i in range(nq)])
+    ref = O.search(Q, R, c32, 4, packed, scale, k, d, tenant_ids=tenants, allow_off=off, allow_ids=ids_allowed)
+    check_topk(ids, sc, ref.ids, ref.scores64, allowed, k, TOL_MMA)
