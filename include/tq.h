@@ -191,6 +191,15 @@ tq_status tq_encode_ex(const float* X, int64_t n, int d, const float* R,
  * tq_encode_check  waits for `stream`, then returns TQ_ETIMEOUT if an encode
  *                with this plan gave up since the plan was built or last
  *                checked (clearing the record), else TQ_OK.
+ * tq_encode_planned_ws  tq_encode_planned with a device workspace, 16-byte
+ *                aligned, of ws_bytes >= tq_encode_workspace(n, d): the rotation
+ *                then runs on the tensor cores in fp16 (about twice TF32's
+ *                rate), again in three products of operands split in two, each
+ *                row of X and R scaled by a power of two first.  fp16 keeps the
+ *                same 10 mantissa bits as TF32, so the error is no larger; the
+ *                calls may land boundary coordinates in different cells.  The
+ *                workspace is free again when the call's work has finished.
+ *                n up to 2^31 - 1024.
  */
 tq_status tq_encode_plan_bytes(int d, size_t* bytes);
 tq_status tq_encode_plan(const float* R, int d, void* plan, size_t plan_bytes, void* stream);
@@ -198,6 +207,12 @@ tq_status tq_encode_planned(const float* X, int64_t n, int d, const void* plan,
                             const float* centroids, const float* boundaries, int bits,
                             int scale_mode, const float* cal_mu, const float* cal_a,
                             uint8_t* codes, float* scale, void* stream);
+tq_status tq_encode_workspace(int64_t n, int d, size_t* bytes);
+tq_status tq_encode_planned_ws(const float* X, int64_t n, int d, const void* plan,
+                               const float* centroids, const float* boundaries, int bits,
+                               int scale_mode, const float* cal_mu, const float* cal_a,
+                               uint8_t* codes, float* scale, void* workspace, size_t ws_bytes,
+                               void* stream);
 tq_status tq_encode_check(const void* plan, void* stream);
 
 /*

@@ -13,7 +13,7 @@ import numpy as np
 
 from ._lib import (MARGINALS, PATHS, SCALE_MODES, TQ_EUNSUPPORTED, TQError, check, load)  # noqa: F401
 
-__all__ = ["codebook", "rotation", "encode", "encode_plan", "encode_plan_bytes", "encode_check", "calibrate", "Filter", "IdMap", "Index", "search", "search_workspace",
+__all__ = ["codebook", "rotation", "encode", "encode_plan", "encode_plan_bytes", "encode_workspace", "encode_check", "calibrate", "Filter", "IdMap", "Index", "search", "search_workspace",
            "search_from_host", "search_host_staging", "search_check", "merge_topk", "set_search_path",
            "profile_events", "row_bytes", "load", "TQError"]
 
@@ -96,11 +96,14 @@ def rotation(d: int, seed: int) -> np.ndarray:
 
 
 def encode(X, R, centroids, boundaries, bits: int, scale_mode: str = "norm",
-           codes=None, scale=None, stream=None, calib=None, plan=None):
+           codes=None, scale=None, stream=None, calib=None, plan=None, workspace=None):
     """tq_encode (tq_encode_ex with a TQ+ calibration `calib` = (mu, a), CUDA
     float32 tensors [d]) on CUDA tensors: returns (codes uint8 [n, d*bits/8],
     scale f32 [n]).  With `plan` (encode_plan(R)) the rotation runs on the
-    tensor cores (tq_encode_planned) and R is not read."""
+    tensor cores (tq_encode_planned_ws) and R is not read; `workspace`
+    (CUDA uint8, encode_workspace(n, d) bytes) may be kept between calls,
+    otherwise one is allocated, or, where it does not fit in device memory, the
+    encoder that needs none runs (tq_encode_planned)."""
     torch = _torch()
     n, d = X.shape
     with _on_stream(stream):
@@ -112,11 +115,24 @@ def encode(X, R, centroids, boundaries, bits: int, scale_mode: str = "norm",
     mu, a = calib if calib is not None else (None, None)
     tail = (_dev_ptr(centroids, "centroids", f32), _dev_ptr(boundaries, "boundaries", f32), bits,
             SCALE_MODES[scale_mode], _dev_ptr(mu, "mu", f32) or None, _dev_ptr(a, "a", f32) or None,
-            _dev_ptr(codes, "codes", torch.uint8), _dev_ptr(scale, "scale", f32), _stream_handle(stream))
+            _dev_ptr(codes, "codes", torch.uint8), _dev_ptr(scale, "scale", f32))
+    handle = _stream_handle(stream)
     if plan is not None:
-        check(load().tq_encode_planned(_dev_ptr(X, "X", f32), n, d, _dev_ptr(plan, "plan", torch.uint8), *tail))
+        need = encode_workspace(n, d)
+        if workspace is None and need is not None:
+            try:
+                with _on_stream(stream):
+                    workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
+            except torch.OutOfMemoryError:
+                pass
+        head = (_dev_ptr(X, "X", f32), n, d, _dev_ptr(plan, "plan", torch.uint8))
+        if workspace is not None:
+            check(load().tq_encode_planned_ws(*head, *tail, _dev_ptr(workspace, "workspace"),
+                                              workspace.numel() * workspace.element_size(), handle))
+        else:
+            check(load().tq_encode_planned(*head, *tail, handle))
     else:
-        check(load().tq_encode_ex(_dev_ptr(X, "X", f32), n, d, _dev_ptr(R, "R", f32), *tail))
+        check(load().tq_encode_ex(_dev_ptr(X, "X", f32), n, d, _dev_ptr(R, "R", f32), *tail, handle))
     return codes, scale
 
 
@@ -128,6 +144,17 @@ def encode_plan_bytes(d: int):
     if st == TQ_EUNSUPPORTED:
         return None
     check(st)
+    return need.value
+
+
+def encode_workspace(n: int, d: int):
+    """tq_encode_workspace: device bytes of scratch for encoding n rows with a
+    plan, or None where that encoder does not apply."""
+    need = C.c_size_t()
+    try:
+        check(load().tq_encode_workspace(n, d, C.byref(need)))
+    except TQError:
+        return None
     return need.value
 
 

@@ -138,21 +138,23 @@ extern "C" tq_status tq_encode_plan(const float* R, int d, void* plan, size_t pl
   return tq::ok();
 }
 
-extern "C" tq_status tq_encode_planned(const float* X, int64_t n, int d, const void* plan,
-                                       const float* centroids, const float* boundaries, int bits,
-                                       int scale_mode, const float* cal_mu, const float* cal_a, uint8_t* codes,
-                                       float* scale, void* stream) {
-  tq_status st = tq::check_common("tq_encode_planned", d, bits);
+namespace tq {
+namespace {
+// The argument checks of the planned encodes.
+tq_status check_planned(const float* X, int64_t n, int d, const void* plan, const float* centroids,
+                        const float* boundaries, int bits, int scale_mode, const float* cal_mu, const float* cal_a,
+                        const uint8_t* codes, const float* scale) {
+  tq_status st = check_common("tq_encode_planned", d, bits);
   if (st != TQ_OK) return st;
-  if (!tq::encode_tc_supported(d))
-    return fail(TQ_EUNSUPPORTED, "tq_encode_planned: d=%d is not a multiple of 32 in [128, %d]", d, tq::kMaxD);
+  if (!encode_tc_supported(d))
+    return fail(TQ_EUNSUPPORTED, "tq_encode_planned: d=%d is not a multiple of 32 in [128, %d]", d, kMaxD);
   if (n < 0 || n > INT32_MAX) return fail(TQ_EINVAL, "tq_encode_planned: n=%lld outside [0, 2^31-1]", (long long)n);
   if (scale_mode != TQ_SCALE_NORM && scale_mode != TQ_SCALE_NONE && scale_mode != TQ_SCALE_UNBIASED)
     return fail(TQ_EINVAL, "tq_encode_planned: unknown scale_mode %d", scale_mode);
-  if (n == 0) return tq::ok();
+  if (n == 0) return TQ_OK;
   if (!X || !plan || !centroids || !boundaries || !codes || !scale)
     return fail(TQ_EINVAL, "tq_encode_planned: NULL device pointer");
-  if (!tq::aligned16(X) || !tq::aligned16(plan) || !tq::aligned16(codes))
+  if (!aligned16(X) || !aligned16(plan) || !aligned16(codes))
     return fail(TQ_EINVAL, "tq_encode_planned: X, plan and codes must be 16-byte aligned");
   if (((uintptr_t)scale & 3u) || ((uintptr_t)centroids & 3u) || ((uintptr_t)boundaries & 3u))
     return fail(TQ_EINVAL, "tq_encode_planned: scale, centroids and boundaries must be 4-byte aligned");
@@ -160,9 +162,52 @@ extern "C" tq_status tq_encode_planned(const float* X, int64_t n, int d, const v
     return fail(TQ_EINVAL, "tq_encode_planned: a TQ+ calibration needs both mu and a");
   if (((uintptr_t)cal_mu & 3u) || ((uintptr_t)cal_a & 3u))
     return fail(TQ_EINVAL, "tq_encode_planned: mu and a must be 4-byte aligned");
+  return TQ_OK;
+}
+}  // namespace
+}  // namespace tq
+
+extern "C" tq_status tq_encode_planned(const float* X, int64_t n, int d, const void* plan,
+                                       const float* centroids, const float* boundaries, int bits,
+                                       int scale_mode, const float* cal_mu, const float* cal_a, uint8_t* codes,
+                                       float* scale, void* stream) {
+  const tq_status st = tq::check_planned(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a, codes,
+                                         scale);
+  if (st != TQ_OK) return st;
+  if (n == 0) return tq::ok();
   const cudaError_t e = tq::launch_encode_tc(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a,
                                              codes, scale, (cudaStream_t)stream);
   if (e != cudaSuccess) return tq::cuda_fail("tq_encode_planned", e);
+  return tq::ok();
+}
+
+extern "C" tq_status tq_encode_workspace(int64_t n, int d, size_t* bytes) {
+  if (!bytes) return fail(TQ_EINVAL, "tq_encode_workspace: NULL bytes");
+  if (n < 0 || n > INT32_MAX - 1024)
+    return fail(TQ_EINVAL, "tq_encode_workspace: n=%lld outside [0, 2^31-1024)", (long long)n);
+  if (!tq::encode_tc_supported(d))
+    return fail(TQ_EUNSUPPORTED, "tq_encode_workspace: d=%d is not a multiple of 32 in [128, %d]", d, tq::kMaxD);
+  *bytes = tq::encode_h_workspace(n, d);
+  return tq::ok();
+}
+
+extern "C" tq_status tq_encode_planned_ws(const float* X, int64_t n, int d, const void* plan,
+                                          const float* centroids, const float* boundaries, int bits,
+                                          int scale_mode, const float* cal_mu, const float* cal_a, uint8_t* codes,
+                                          float* scale, void* workspace, size_t ws_bytes, void* stream) {
+  const tq_status st = tq::check_planned(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a, codes,
+                                         scale);
+  if (st != TQ_OK) return st;
+  if (n == 0) return tq::ok();
+  size_t need = 0;
+  const tq_status ws = tq_encode_workspace(n, d, &need);
+  if (ws != TQ_OK) return ws;
+  if (!workspace || !tq::aligned16(workspace))
+    return fail(TQ_EINVAL, "tq_encode_planned_ws: the workspace must be 16-byte aligned device memory");
+  if (ws_bytes < need) return fail(TQ_EINVAL, "tq_encode_planned_ws: workspace of %zu bytes, %zu needed", ws_bytes, need);
+  const cudaError_t e = tq::launch_encode_h(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a,
+                                            codes, scale, workspace, (cudaStream_t)stream);
+  if (e != cudaSuccess) return tq::cuda_fail("tq_encode_planned_ws", e);
   return tq::ok();
 }
 

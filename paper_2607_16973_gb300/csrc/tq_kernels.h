@@ -36,6 +36,13 @@ cudaError_t launch_encode_tc(const float* X, int64_t n, int d, const void* plan,
                              const float* boundaries, int bits, int scale_mode, const float* cal_mu,
                              const float* cal_a, uint8_t* codes, float* scale, cudaStream_t s);
 
+// The same in fp16 (three products of operands split in two, rows scaled by
+// powers of two), with a workspace of encode_h_workspace(n, d) bytes.
+size_t encode_h_workspace(int64_t n, int d);
+cudaError_t launch_encode_h(const float* X, int64_t n, int d, const void* plan, const float* centroids,
+                            const float* boundaries, int bits, int scale_mode, const float* cal_mu,
+                            const float* cal_a, uint8_t* codes, float* scale, void* ws, cudaStream_t s);
+
 // Query rotation on the tensor cores for batches of kRotTcMinBatch or more
 // (d as for the tensor-core encoder): q' = R q in TF32 with the three-product
 // split, the contraction split over rotate_tc_splits(nq, d) CTAs whose
