@@ -288,7 +288,13 @@ k_rotate_gemm(const float* __restrict__ Q, int64_t nq, int d, const float* __res
 }
 
 // Q' = Q R^T for groups of NQ <= 8 queries: one warp per output coordinate,
-// R read once per group.
+// R read once per group.  Bound by R's way from HBM (9.4 MB at d = 1536, 1.4 us)
+// and by latency: R (d*d*4 bytes) is usually evicted from L2 by the corpus
+// stream between searches, so a lane issues its row loads (up to 16, or 8)
+// before using any of them, and the queries' values (L1 hits: every
+// warp of an SM reads the same ones) come in batches of 16 loads a lane, not one
+// by one between the products: eight queries at d = 1536 42 -> 13 us, cold.  The
+// order of the sums is the same for every NQ.
 template <int NQ>
 __global__ void __launch_bounds__(256)
 k_rotate_gemv(const float* __restrict__ Q, int64_t nq, int d, const float* __restrict__ R, float* __restrict__ out,
@@ -307,10 +313,8 @@ k_rotate_gemv(const float* __restrict__ Q, int64_t nq, int d, const float* __res
   for (int q = 0; q < NQ; ++q) acc[q] = 0.f;
   const float4* r4 = reinterpret_cast<const float4*>(R + (int64_t)i * d);
   const int d4 = d / 4;
-  // R (d*d*4 bytes) is usually evicted from L2 by the corpus stream between
-  // searches, so a lane issues all its row loads (16 for d = 2048) before
-  // using any of them
-  constexpr int RL = 16;
+  constexpr int RL = NQ <= 2 ? 16 : 8;  // row loads in flight (two blocks of 8 warps per SM need 128 registers)
+  constexpr int U = NQ == 1 ? 16 : NQ == 2 ? 8 : NQ <= 4 ? 4 : 2;  // of them per batch of query loads
   for (int j0 = lane; j0 < d4; j0 += 32 * RL) {
     float4 rv[RL];
 #pragma unroll
@@ -319,17 +323,27 @@ k_rotate_gemv(const float* __restrict__ Q, int64_t nq, int d, const float* __res
       rv[t] = j < d4 ? __ldg(r4 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
-    for (int t = 0; t < RL; ++t) {
-      const int j = j0 + 32 * t;
-      if (j >= d4) break;
+    for (int t0 = 0; t0 < RL; t0 += U) {
+      if (j0 - lane + 32 * t0 >= d4) break;  // the same for the whole warp
+      float4 qv[U][NQ];
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        if (q >= nqg) break;
-        const float4 qv = __ldg(reinterpret_cast<const float4*>(Q + (int64_t)q * d) + j);
-        acc[q] = fmaf(rv[t].x, qv.x, acc[q]);
-        acc[q] = fmaf(rv[t].y, qv.y, acc[q]);
-        acc[q] = fmaf(rv[t].z, qv.z, acc[q]);
-        acc[q] = fmaf(rv[t].w, qv.w, acc[q]);
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {  // (a short group's missing queries repeat its last)
+          const int j = min(j0 + 32 * (t0 + u), d4 - 1);
+          qv[u][q] = __ldg(reinterpret_cast<const float4*>(Q + (int64_t)min(q, nqg - 1) * d) + j);
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (j0 + 32 * (t0 + u) >= d4) break;
+        const float4 r = rv[t0 + u];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          acc[q] = fmaf(r.x, qv[u][q].x, acc[q]);
+          acc[q] = fmaf(r.y, qv[u][q].y, acc[q]);
+          acc[q] = fmaf(r.z, qv[u][q].z, acc[q]);
+          acc[q] = fmaf(r.w, qv[u][q].w, acc[q]);
+        }
       }
     }
   }
