@@ -32,15 +32,16 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 struct SearchPlan {
   int grid_lut = 1, grid_mma = 0, grid_fold = 0, grid_tm = 0;
   size_t off_status = 0, off_cnt = 0, off_bias = 0, off_gate = 0, off_lows = 0, off_rot = 0, off_part = 0, off_allow = 0, off_mask = 0,
-         off_qpack = 0, off_cs = 0, off_ci = 0, total = 0;
+         off_qpack = 0, off_lists = 0, off_cs = 0, off_ci = 0, total = 0;
+  int64_t n_cnt = 0;    // words the rotation zeroes: merge counters, thresholds, the force word, list heads
   bool rot_tc = false;  // the query rotation runs on the tensor cores
 };
 
 // Workspace layout (both scan paths): status word | merge counters (one per
-// query, and the small-batch scan's thresholds and force word) | its gates (one per
+// query, and the tensor-core scans' thresholds, force word and list heads) | its gates (one per
 // query) and list bounds (two per query and CTA) | TQ+ query terms (one per query) | rotated queries | partial
 // rotations (tensor-core rotation) | allow bitmaps | block masks | fp16 query
-// tiles (tensor-core scan) | candidate scores | ids.
+// tiles and list scratch (tensor-core scan) | candidate scores | ids.
 SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_filter* filter) {
   SearchPlan p;
   p.grid_lut = scan_lut_grid_x(nq, n, k, bits, d);
@@ -55,7 +56,8 @@ SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_f
   p.off_status = off;
   off = align_up(off + sizeof(int));
   p.off_cnt = off;
-  off = align_up(off + ((size_t)2 * nq + 1) * sizeof(int));
+  p.n_cnt = 2 * nq + 1 + (int64_t)p.grid_mma * nq;
+  off = align_up(off + (size_t)p.n_cnt * sizeof(int));
   p.off_gate = off;
   if (tm) off = align_up(off + (size_t)nq * sizeof(int));
   p.off_lows = off;
@@ -73,6 +75,8 @@ SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_f
   if (filter) off = align_up(off + (size_t)nq * filter_mask_words(filter->f) * sizeof(uint32_t));
   p.off_qpack = off;
   if (mma) off = align_up(off + mma_qpack_bytes(nq, d));
+  p.off_lists = off;
+  if (mma) off = align_up(off + mma_list_bytes(nq, bits, k, p.grid_mma));
   p.off_cs = off;
   off = align_up(off + (size_t)nq * per_query * sizeof(float));
   p.off_ci = off;
@@ -506,8 +510,8 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
   int* force = counters + 2 * nq;
   // the rotation also clears the status word and zeroes the counters, thresholds and the force word
   cudaError_t e = p.rot_tc ? tq::launch_rotate_tc(Q, nq, d, R, qrot, reinterpret_cast<float*>(ws + p.off_part),
-                                                  status, counters, 2 * nq + 1, s)
-                           : tq::launch_rotate(Q, nq, d, R, qrot, status, counters, 2 * nq + 1, s);
+                                                  status, counters, p.n_cnt, s)
+                           : tq::launch_rotate(Q, nq, d, R, qrot, status, counters, p.n_cnt, s);
   if (e == cudaSuccess && cal_mu) e = tq::launch_calib_query(qrot, nq, d, cal_mu, cal_a, bias, s);
   if (use_tm) {
     float* lows = reinterpret_cast<float*>(ws + p.off_lows);
@@ -533,7 +537,9 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
     if (e == cudaSuccess)
       e = tq::launch_scan_mma(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
                               filter ? filter->f.dense : nullptr, allow, filter ? filter->f.words : 0, bias, k,
-                              p.grid_mma, ws + p.off_qpack, cs, ci, status, s, (cudaEvent_t)tq::profile_start(),
+                              p.grid_mma, ws + p.off_qpack, cs, ci, status, gth,
+                              reinterpret_cast<uint32_t*>(counters + 2 * nq + 1),
+                              reinterpret_cast<uint64_t*>(ws + p.off_lists), s, (cudaEvent_t)tq::profile_start(),
                               (cudaEvent_t)tq::profile_stop());
     if (e == cudaSuccess) e = tq::launch_merge(cs, ci, nq, p.grid_mma * k, k, ext_ids, out_ids, out_scores, s);
   } else {

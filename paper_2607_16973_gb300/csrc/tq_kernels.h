@@ -132,15 +132,18 @@ cudaError_t launch_merge_global(const float* cand_s, const int64_t* cand_i, int6
 
 // Tensor-core decode-GEMM scan (bits 2, 4, 8; k <= kMaxKMma).  With
 // allow_bits [nq * words] (and the filter's dense tenant index) a vector whose
-// tenant the query does not allow never enters its list.
+// tenant the query does not allow never enters its list.  `gth` [nq] and
+// `heads` [grid_x][nq], zeroed by the query rotation: thresholds and best scores
+// that the CTAs of a query share.
 bool mma_supported(int bits, int d, int k);
 int scan_mma_grid_x(int64_t nq, int64_t n, int k, int bits);
 size_t mma_qpack_bytes(int64_t nq, int d);
+size_t mma_list_bytes(int64_t nq, int bits, int k, int grid_x);  // the `lists` scratch: a list per query and CTA
 cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
                             const uint8_t* codes, const float* scale, int64_t n, const uint32_t* del,
                             const uint32_t* dense, const uint32_t* allow_bits, int words, const float* bias,
-                            int k, int grid_x, void* qpack, float* cand_s, int32_t* cand_i, int* err, cudaStream_t s,
-                            cudaEvent_t ev0, cudaEvent_t ev1);
+                            int k, int grid_x, void* qpack, float* cand_s, int32_t* cand_i, int* err, uint32_t* gth,
+                            uint32_t* heads, uint64_t* lists, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1);
 
 // Small-batch tensor-core scan of 4-bit codes (k_scan_tm).  With `bound` it is
 // the first half of an exact float32 search of at most 16 queries: every CTA

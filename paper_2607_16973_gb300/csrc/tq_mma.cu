@@ -92,12 +92,25 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b,
       ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc<N>()), "r"(accumulate));
 }
 
-__device__ __forceinline__ bool better(float s1, int i1, float s2, int i2) {
-  return s1 > s2 || (s1 == s2 && i1 < i2);
+// Scores as unsigned integers of the same order (0 below every score's), for
+// the thresholds that the CTAs of a query share.
+__device__ __forceinline__ uint32_t order_bits(float s) {
+  const uint32_t b = __float_as_uint(s + 0.0f);
+  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float ordered(uint32_t o) {
+  return __uint_as_float(o & 0x80000000u ? o ^ 0x80000000u : ~o);
 }
 
+// A score and its row as one key, larger = better (score descending, id ascending).
+__device__ __forceinline__ uint64_t rank_key(float s, int id) {
+  return ((uint64_t)order_bits(s) << 32) | (uint32_t)~id;
+}
+__device__ __forceinline__ float key_score(uint64_t key) { return ordered((uint32_t)(key >> 32)); }
+__device__ __forceinline__ int key_id(uint64_t key) { return (int)~(uint32_t)key; }
+
 struct MmaSmem {
-  uint32_t a, b, raw, tab, scale, dense, lists_s, lists_i, bars, total;
+  uint32_t a, b, raw, tab, scale, dense, bars, total;
 };
 
 template <int BITS>
@@ -121,7 +134,7 @@ __host__ __device__ inline int tile_sub(int bits, int rr) {
 // Shared-memory plan for QT query tiles per CTA, `cst` raw code stages and
 // `ast` query stages.
 template <int BITS, int QT>
-__host__ __device__ inline MmaSmem mma_smem_layout(int k, int cst, int ast, int rr, int ng) {
+__host__ __device__ inline MmaSmem mma_smem_layout(int cst, int ast, int rr, int ng) {
   MmaSmem L{};
   uint32_t off = 0;
   L.a = off;
@@ -136,10 +149,6 @@ __host__ __device__ inline MmaSmem mma_smem_layout(int k, int cst, int ast, int 
   off += tile_n<QT>() * 4;
   L.dense = off;  // tenant index of each vector of the tile (filtered searches)
   off += tile_n<QT>() * 4;
-  L.lists_s = off;
-  off += (uint32_t)QT * k * MMA_M * 4;
-  L.lists_i = off;
-  off += (uint32_t)QT * k * MMA_M * 4;
   off = (off + 15) & ~15u;
   L.bars = off;
   off += 48 * 8;
@@ -174,7 +183,7 @@ constexpr int MIN_PREFETCH_KB = 6;  // K-blocks of codes in flight (HBM latency)
 // groups as the role layout has (all of them able to run), with at least
 // MIN_PREFETCH_KB K-blocks of codes in flight, then deeper rings.
 template <int BITS>
-MmaPlan mma_plan(int64_t nq, int k) {
+MmaPlan mma_plan(int64_t nq) {
   MmaPlan best;
   // first pass as above; the second relaxes the prefetch floor and allows
   // fewer groups (large k at 8 bits needs the room for its lists)
@@ -188,8 +197,8 @@ MmaPlan mma_plan(int64_t nq, int k) {
           for (int ast = 3; ast >= 2; --ast) {
             for (int cst = MAX_CST; cst >= 2; --cst) {
               if (cst * sub < min_pf || active_groups(ng, sub, cst) != ng) continue;
-              const uint32_t need = qt == 2 ? mma_smem_layout<BITS, 2>(k, cst, ast, rr, ng).total
-                                            : mma_smem_layout<BITS, 1>(k, cst, ast, rr, ng).total;
+              const uint32_t need = qt == 2 ? mma_smem_layout<BITS, 2>(cst, ast, rr, ng).total
+                                            : mma_smem_layout<BITS, 1>(cst, ast, rr, ng).total;
               if (need <= kMaxDynSmem) {
                 best.qt = qt;
                 best.cst = cst;
@@ -243,7 +252,8 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
            const uint32_t* __restrict__ del, const uint32_t* __restrict__ dense,
            const uint32_t* __restrict__ allow_bits, int words, const float* __restrict__ bias, int n, int nq,
            int d, int k, int cst, int ast, int rr, int sub, int ng, int gact, float* __restrict__ cand_s,
-           int* __restrict__ cand_i, int* __restrict__ err) {
+           int* __restrict__ cand_i, int* __restrict__ err, uint32_t* __restrict__ gth,
+           uint32_t* heads, uint64_t* __restrict__ lists) {
   constexpr int RAWB = raw_bytes_per_row<BITS>();
   // A code tile carries `sub` consecutive K-blocks of 256 rows: rows of
   // sub*RAWB bytes (128 B, one full line, when d allows), stored with the
@@ -261,14 +271,12 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
   // pointer arithmetic on the shared array (not an integer round trip) keeps
   // every access below a shared-memory access
   unsigned char* base = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
-  const MmaSmem L = mma_smem_layout<BITS, QT>(k, cst, ast, rr, ng);
+  const MmaSmem L = mma_smem_layout<BITS, QT>(cst, ast, rr, ng);
   unsigned char* sA = base + L.a;
   unsigned char* sB = base + L.b;
   unsigned char* sRaw = base + L.raw;
   float* sScale = reinterpret_cast<float*>(base + L.scale);
   uint32_t* sDense = reinterpret_cast<uint32_t*>(base + L.dense);
-  float* lst_s = reinterpret_cast<float*>(base + L.lists_s);
-  int* lst_i = reinterpret_cast<int*>(base + L.lists_i);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + L.bars);
   uint64_t* cfull = bars;                      // [MAX_CST] code tile landed
   uint64_t* cempty = bars + 8;                 // [MAX_CST] code tile decoded (stage free)
@@ -509,42 +517,38 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
     // a filtered search: this query's allow bitmap over the dense tenant index
     const uint32_t* ab = allow_bits && q < nq ? allow_bits + (size_t)q * words : nullptr;
     const float bq = bias && q < nq ? bias[q] : 0.f;  // a TQ+ index's per-query term (else 0)
-    float* ls = lst_s + jsel * k * MMA_M;
-    int* li = lst_i + jsel * k * MMA_M;
-    if (mine) {
-      for (int i = 0; i < k; ++i) {
-        ls[i * MMA_M + row] = -INFINITY;
-        li[i * MMA_M + row] = INT_MAX;
-      }
-    }
+    // This query's k best so far: keys in no order, and the worst of them.  They
+    // live in global memory (L1 and L2), not in shared memory, whose room they
+    // took from the decoded tiles' stages (k = 10: two decoder groups instead of
+    // three), and are not kept sorted: a new entry replaces the worst and the
+    // list is read once, k independent loads, for the next worst.  Shifting a
+    // sorted list entry by entry cost about 60 cycles each: 300 of the 430 us of
+    // 50 queries, k = 20, over 300,001 x 1024.
+    uint64_t* lst = lists + (((size_t)blockIdx.y * gridDim.x + blockIdx.x) * QT + jsel) * k * MMA_M + row;
+    uint64_t worst = 0;  // 0: not full yet
+    int cnt = 0, wslot = 0;
     float th_s = -INFINITY;
-    int th_i = INT_MAX;
+    // k vectors of the corpus score at least th_g (the best threshold any CTA
+    // has published): what is below cannot be among the k best
+    float th_g = -INFINITY, th = -INFINITY;  // th = max(th_s, th_g)
+    uint32_t published = 0, head = 0, head_out = 0;  // head: the best score so far (order_bits)
     float ps0 = 0.f, ps1 = 0.f, ps2 = 0.f, ps3 = 0.f;  // parked candidates of the current tile
     int pi0 = 0, pi1 = 0, pi2 = 0, pi3 = 0, npark = 0;
-    // Inserts (sc, v) into this thread's sorted list if it beats entry
-    // k-1: walk up while the entry above is worse, shifting it down; the
-    // new entry k-1 is the first one shifted, or (sc, v) if nothing moves.
     auto insert = [&](float sc, int v) {
-      if (!better(sc, v, th_s, th_i)) return;
-      float nts = sc;
-      int nti = v;
-      int pos = k - 1;
-      while (pos > 0) {
-        const float as = ls[(pos - 1) * MMA_M + row];
-        const int ai = li[(pos - 1) * MMA_M + row];
-        if (!better(sc, v, as, ai)) break;
-        ls[pos * MMA_M + row] = as;
-        li[pos * MMA_M + row] = ai;
-        if (pos == k - 1) {
-          nts = as;
-          nti = ai;
-        }
-        --pos;
+      const uint64_t key = rank_key(sc, v);
+      if (key <= worst) return;
+      lst[(cnt < k ? cnt : wslot) * MMA_M] = key;
+      head = max(head, (uint32_t)(key >> 32));
+      if (cnt < k) ++cnt;
+      if (cnt < k) return;
+      worst = ~0ull;
+#pragma unroll 4
+      for (int i = 0; i < k; ++i) {
+        const uint64_t o = lst[i * MMA_M];
+        wslot = o < worst ? i : wslot;
+        worst = o < worst ? o : worst;
       }
-      ls[pos * MMA_M + row] = sc;
-      li[pos * MMA_M + row] = v;
-      th_s = nts;
-      th_i = nti;
+      th_s = key_score(worst);
     };
     for (int tile_i = 0; tile_i < my_tiles; ++tile_i) {
       const int t = blockIdx.x + tile_i * gridDim.x;
@@ -556,6 +560,34 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
         const int v = v0 + j;
         sScale[j] = v < n ? (scale ? scale[v] : 1.0f) : 0.0f;
         if (allow_bits) sDense[j] = v < n ? __ldg(dense + v) : 0u;
+      }
+      const uint32_t shared_th = mine && q < nq ? __ldcg(gth + q) : 0u;
+      if ((tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= 8 && k <= 32 &&
+          (int)gridDim.x >= k && mine && q < nq) {
+        // Every CTA publishes its best score for the query.  The k-th best of
+        // the maxima of 32 groups of CTAs is reached by k vectors; with all
+        // CTAs' rows behind it, few vectors of a tile reach it (a CTA's own
+        // list is beaten by k / i vectors of its tile i).  It costs about 5 us, so
+        // not for a small k: 300,001 x 1024, 50 queries: k = 20 281 -> 238 us, k = 5
+        // 153 -> 174; 999,000 x 1536, 256 queries: k = 10 809 -> 744, k = 5 731 -> 722.
+        uint32_t g[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) g[i] = 0;
+#pragma unroll 1
+        for (int c = 0; c < (int)gridDim.x; c += 32)
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c + i < (int)gridDim.x) g[i] = max(g[i], __ldcg(heads + (size_t)(c + i) * nq + q));
+        uint32_t b = 0;
+#pragma unroll 1
+        for (int bit = 31; bit >= 12; --bit) {  // (rounded down: 12 mantissa bits do)
+          const uint32_t up = b | (1u << bit);
+          int have = 0;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) have += g[i] >= up ? 1 : 0;
+          b = have >= k ? up : b;
+        }
+        if (b) th_g = fmaxf(th_g, ordered(b));
       }
       asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
       // all epilogue warps take the same decision, so none is left at bar.sync
@@ -571,6 +603,47 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       tc_fence_after();
       if (mine) {
         const uint32_t tb = tmem + ((uint32_t)(32 * e) << 16) + (uint32_t)((set * QT + jsel) * NT);
+        if (shared_th) th_g = fmaxf(th_g, ordered(shared_th));
+        if (tile_i == 0 && !allow_bits && n - v0 >= NT) {
+          // The first tile's vectors all pass an empty list's threshold, and
+          // taking up to 256 of them into the list one by one took longer than
+          // many tiles' MMAs (k = 20: about 100 us).  So the list first takes
+          // the maxima of groups of 8 columns (4 for k > 32): k of those are
+          // distinct vectors, so their k-th best is a first threshold, which
+          // about k vectors of the tile reach.
+          const bool fine = k > 32;
+#pragma unroll 1
+          for (int c0 = 0; c0 < NT; c0 += 16) {
+            uint32_t r[16];
+            tmem_ld16_issue(tb + (uint32_t)c0, r);
+            tmem_wait16(r);
+            if (q >= nq) continue;
+            const uint32_t dead = del ? __ldg(del + ((v0 + c0) >> 5)) >> (c0 & 16) : 0u;
+            float m4[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float4 s4 = *reinterpret_cast<const float4*>(sScale + c0 + 4 * j);
+              const float x[4] = {(__uint_as_float(r[4 * j]) + bq) * s4.x, (__uint_as_float(r[4 * j + 1]) + bq) * s4.y,
+                                  (__uint_as_float(r[4 * j + 2]) + bq) * s4.z,
+                                  (__uint_as_float(r[4 * j + 3]) + bq) * s4.w};
+              m4[j] = -INFINITY;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) m4[j] = fmaxf(m4[j], (dead >> (4 * j + i)) & 1u ? -INFINITY : x[i]);
+            }
+#pragma unroll 1
+            for (int j = fine ? 0 : 1; j < 4; j += fine ? 1 : 2) {
+              const float pair = fmaxf(j == 1 ? m4[0] : m4[2], j == 1 ? m4[1] : m4[3]);
+              insert(fine ? (j == 0 ? m4[0] : j == 1 ? m4[1] : j == 2 ? m4[2] : m4[3]) : pair, c0 + 4 * j);
+            }
+          }
+          th_g = fmaxf(th_g, th_s);
+          worst = 0;
+          cnt = 0;
+          head = 0;
+          th_s = -INFINITY;
+          __syncwarp();
+        }
+        th = fmaxf(th_s, th_g);
         // one 16-column chunk: scale, flag the scores that may enter the list
         // (branch-free); flagged ones (rare after the first tiles) are parked
         // in registers and inserted after the accumulator is released, so the
@@ -591,10 +664,10 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
             r[jj + 1] = __float_as_uint(x.y);
             r[jj + 2] = __float_as_uint(y.x);
             r[jj + 3] = __float_as_uint(y.y);
-            m |= (x.x >= th_s ? 1u : 0u) << jj;
-            m |= (x.y >= th_s ? 1u : 0u) << (jj + 1);
-            m |= (y.x >= th_s ? 1u : 0u) << (jj + 2);
-            m |= (y.y >= th_s ? 1u : 0u) << (jj + 3);
+            m |= (x.x >= th ? 1u : 0u) << jj;
+            m |= (x.y >= th ? 1u : 0u) << (jj + 1);
+            m |= (y.x >= th ? 1u : 0u) << (jj + 2);
+            m |= (y.y >= th ? 1u : 0u) << (jj + 3);
           }
           if (valid < 16) m &= valid > 0 ? (1u << valid) - 1u : 0u;
           while (m) {
@@ -604,7 +677,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
 #pragma unroll
             for (int t = 0; t < 16; ++t) sc = t == jj ? __uint_as_float(r[t]) : sc;
             const int v = v0 + c0 + jj;
-            if (!better(sc, v, th_s, th_i)) continue;
+            if (rank_key(sc, v) <= worst) continue;
             if (del && ((__ldg(del + (v >> 5)) >> (v & 31)) & 1u)) continue;  // deleted row
             if (ab) {  // tenant not allowed: never enters the list (Sec. III-B)
               const uint32_t t = sDense[c0 + jj];
@@ -622,6 +695,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
               ++npark;
             } else {
               insert(sc, v);
+              th = fmaxf(th_s, th_g);
             }
           }
         };
@@ -649,13 +723,27 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       if (npark > 2) insert(ps2, pi2);
       if (npark > 3) insert(ps3, pi3);
       npark = 0;
+      if (mine && q < nq && worst && th_s >= th_g) {  // a full list's k-th best
+        const uint32_t b = order_bits(th_s);
+        if (b > published && b > shared_th) atomicMax(gth + q, b);
+        published = b;
+      }
+      if (mine && q < nq && head > head_out) heads[(size_t)blockIdx.x * nq + q] = head_out = head;
       asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
     }
     if (mine && q < nq) {
-      for (int i = 0; i < k; ++i) {
-        const size_t o = ((size_t)q * gridDim.x + blockIdx.x) * k + i;
-        cand_s[o] = ls[i * MMA_M + row];
-        cand_i[o] = li[i * MMA_M + row];
+      uint64_t last = ~0ull;  // written best first: each round takes the best key below the last one's
+      for (int r = 0; r < k; ++r) {
+        uint64_t best = 0;
+#pragma unroll 4
+        for (int i = 0; i < cnt; ++i) {
+          const uint64_t o = lst[i * MMA_M];
+          best = o < last && o > best ? o : best;
+        }
+        const size_t o = ((size_t)q * gridDim.x + blockIdx.x) * k + r;
+        cand_s[o] = best ? key_score(best) : -INFINITY;
+        cand_i[o] = best ? key_id(best) : INT_MAX;
+        last = best;
       }
     }
   }
@@ -691,7 +779,7 @@ template <int BITS, int QT>
 cudaError_t launch_typed(const MmaPlan& P, const CUtensorMap& map, const __half* qpack, const float* centroids,
                          const float* scale, const uint32_t* del, const uint32_t* dense, const uint32_t* allow,
                          int words, const float* bias, int n, int nq, int d, int k, int sub, int grid_x, float* cs,
-                         int* ci, int* err, cudaStream_t s) {
+                         int* ci, int* err, uint32_t* gth, uint32_t* heads, uint64_t* lists, cudaStream_t s) {
   const int gact = active_groups(P.ng, sub, P.cst);
   cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_scan_mma<BITS, QT>), (int)P.smem);
   if (e != cudaSuccess) return e;
@@ -699,13 +787,13 @@ cudaError_t launch_typed(const MmaPlan& P, const CUtensorMap& map, const __half*
   const dim3 grid((unsigned)grid_x, (unsigned)((nqt + QT - 1) / QT));
   k_scan_mma<BITS, QT><<<grid, NTHREADS, P.smem, s>>>(map, qpack, centroids, scale, del, dense, allow, words, bias,
                                                          n, nq, d, k, P.cst, P.ast, P.rr, sub, P.ng, gact, cs, ci,
-                                                         err);
+                                                         err, gth, heads, lists);
   return cudaGetLastError();
 }
 
-MmaPlan plan_for(int bits, int64_t nq, int k) {
-  return bits == 2 ? mma_plan<2>(nq, k) : bits == 3 ? mma_plan<3>(nq, k) : bits == 4 ? mma_plan<4>(nq, k)
-                                                                           : mma_plan<8>(nq, k);
+MmaPlan plan_for(int bits, int64_t nq) {
+  return bits == 2 ? mma_plan<2>(nq) : bits == 3 ? mma_plan<3>(nq) : bits == 4 ? mma_plan<4>(nq)
+                                                                           : mma_plan<8>(nq);
 }
 
 }  // namespace
@@ -713,12 +801,12 @@ MmaPlan plan_for(int bits, int64_t nq, int k) {
 bool mma_supported(int bits, int d, int k) {
   // 3-bit code tiles carry an even number of K-blocks: d a multiple of 128
   return (bits == 2 || bits == 3 || bits == 4 || bits == 8) && d % (bits == 3 ? 2 * KB : KB) == 0 && k >= 1 &&
-         k <= kMaxKMma && plan_for(bits, 1, k).smem != 0;
+         k <= kMaxKMma && plan_for(bits, 1).smem != 0;
 }
 
 int scan_mma_grid_x(int64_t nq, int64_t n, int k, int bits) {
   const int64_t qtiles = (nq + MMA_M - 1) / MMA_M;
-  const int qt = plan_for(bits, nq, k).qt;
+  const int qt = plan_for(bits, nq).qt;
   const int64_t groups = (qtiles + qt - 1) / qt;
   const int64_t ntiles = (n + MMA_N - 1) / MMA_N;
   int64_t gx = ((int64_t)device_sm_count() + groups - 1) / groups;
@@ -731,16 +819,23 @@ size_t mma_qpack_bytes(int64_t nq, int d) {
   return (size_t)((nq + MMA_M - 1) / MMA_M) * (d / KB) * A_BYTES;
 }
 
+size_t mma_list_bytes(int64_t nq, int bits, int k, int grid_x) {
+  const int qt = plan_for(bits, nq).qt;
+  const int64_t groups = ((nq + MMA_M - 1) / MMA_M + qt - 1) / qt;
+  return (size_t)groups * grid_x * qt * k * MMA_M * sizeof(uint64_t);
+}
+
 cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
                             const uint8_t* codes, const float* scale, int64_t n, const uint32_t* del,
                             const uint32_t* dense, const uint32_t* allow_bits, int words, const float* bias,
-                            int k, int grid_x, void* qpack, float* cand_s, int32_t* cand_i, int* err, cudaStream_t s,
+                            int k, int grid_x, void* qpack, float* cand_s, int32_t* cand_i, int* err, uint32_t* gth,
+                            uint32_t* heads, uint64_t* lists, cudaStream_t s,
                             cudaEvent_t ev0, cudaEvent_t ev1) {
   if (nq == 0) return cudaSuccess;
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
   if (!enc) return cudaErrorNotSupported;
   const int rawb = KB * bits / 8;
-  const MmaPlan P = plan_for(bits, nq, k);
+  const MmaPlan P = plan_for(bits, nq);
   if (P.smem == 0) return cudaErrorInvalidValue;
   // K-blocks per code tile: up to P.rr bytes of each row, dividing the row's K-blocks
   const int kblocks = d / KB;
@@ -766,9 +861,9 @@ cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* c
 #define TQ_MMA_CASE(B)                                                                                \
   case B:                                                                                             \
     e = P.qt == 2 ? launch_typed<B, 2>(P, map, qp, centroids, scale, del, dense, allow_bits, words, bias, \
-                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, s)        \
+                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, gth, heads, lists, s)        \
                   : launch_typed<B, 1>(P, map, qp, centroids, scale, del, dense, allow_bits, words, bias, \
-                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, s);       \
+                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, gth, heads, lists, s);       \
     break;
   switch (bits) {
     TQ_MMA_CASE(2)
