@@ -543,8 +543,7 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
                               (cudaEvent_t)tq::profile_stop());
     if (e == cudaSuccess) e = tq::launch_merge(cs, ci, nq, p.grid_mma * k, k, ext_ids, out_ids, out_scores, s);
   } else {
-    if (e == cudaSuccess && filter) e = tq::launch_allow_bits(filter->f, allow_off, allow_tenants, nq, allow, s);
-    if (e == cudaSuccess && filter) e = tq::launch_block_mask(filter->f, allow, nq, bmask, s);
+    if (e == cudaSuccess && filter) e = tq::launch_filter_prep(filter->f, allow_off, allow_tenants, nq, allow, bmask, s);
     if (e == cudaSuccess && use_fold)
       e = tq::launch_scan_fold(qrot, nq, d, centroids, codes, scale, n, deleted, filter ? &filter->f : nullptr,
                                allow, bmask, k, p.grid_fold, cs, ci, status, counters, ext_ids, out_ids,

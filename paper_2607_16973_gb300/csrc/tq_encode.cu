@@ -330,8 +330,9 @@ k_rotate_gemv(const float* __restrict__ Q, int64_t nq, int d, const float* __res
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {  // (a short group's missing queries repeat its last)
-          const int j = min(j0 + 32 * (t0 + u), d4 - 1);
-          qv[u][q] = __ldg(reinterpret_cast<const float4*>(Q + (int64_t)min(q, nqg - 1) * d) + j);
+          const int j = j0 + 32 * (t0 + u);
+          qv[u][q] = j < d4 ? __ldg(reinterpret_cast<const float4*>(Q + (int64_t)min(q, nqg - 1) * d) + j)
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
       for (int u = 0; u < U; ++u) {

@@ -114,11 +114,12 @@ cudaError_t launch_scan_fold(const float* qrot, int64_t nq, int d, const float* 
                              float* out_scores, const float* bias, cudaStream_t s, cudaEvent_t ev0,
                              cudaEvent_t ev1);
 
-// Per-query bitmap over the filter's blocks: bit b set when block b holds a
-// tenant the query allows.  out [nq * filter_mask_words(f)].
+// Both filter inputs of a lookup scan: the queries' allow bitmaps (as
+// launch_allow_bits) and, per query, a bitmap over the filter's blocks: bit b set
+// when block b holds a tenant the query allows.  mask [nq * filter_mask_words(f)].
 int filter_mask_words(const FilterDev& f);
-cudaError_t launch_block_mask(const FilterDev& f, const uint32_t* allow, int64_t nq, uint32_t* mask,
-                              cudaStream_t s);
+cudaError_t launch_filter_prep(const FilterDev& f, const int64_t* allow_off, const uint32_t* allow_tenants,
+                               int64_t nq, uint32_t* allow, uint32_t* mask, cudaStream_t s);
 
 // Final merge of per-CTA candidates into sorted top-k; with `ext` (nullable)
 // the rows are written as ext[row].

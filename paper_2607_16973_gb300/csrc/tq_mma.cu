@@ -531,20 +531,24 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
     // k vectors of the corpus score at least th_g (the best threshold any CTA
     // has published): what is below cannot be among the k best
     float th_g = -INFINITY, th = -INFINITY;  // th = max(th_s, th_g)
-    uint32_t published = 0, head = 0, head_out = 0;  // head: the best score so far (order_bits)
     float ps0 = 0.f, ps1 = 0.f, ps2 = 0.f, ps3 = 0.f;  // parked candidates of the current tile
     int pi0 = 0, pi1 = 0, pi2 = 0, pi3 = 0, npark = 0;
+    // tiles before which the CTAs' best scores are read, and after whose
+    // predecessors they are published
+    auto heads_turn = [&](int tile_i) {
+      return (tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= 8 && k <= 32 && (int)gridDim.x >= k;
+    };
     auto insert = [&](float sc, int v) {
       const uint64_t key = rank_key(sc, v);
       if (key <= worst) return;
-      lst[(cnt < k ? cnt : wslot) * MMA_M] = key;
-      head = max(head, (uint32_t)(key >> 32));
+      const int slot = cnt < k ? cnt : wslot;
+      lst[slot * MMA_M] = key;
       if (cnt < k) ++cnt;
       if (cnt < k) return;
       worst = ~0ull;
 #pragma unroll 4
       for (int i = 0; i < k; ++i) {
-        const uint64_t o = lst[i * MMA_M];
+        const uint64_t o = i == slot ? key : lst[i * MMA_M];  // (not waiting for the store)
         wslot = o < worst ? i : wslot;
         worst = o < worst ? o : worst;
       }
@@ -562,9 +566,8 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
         if (allow_bits) sDense[j] = v < n ? __ldg(dense + v) : 0u;
       }
       const uint32_t shared_th = mine && q < nq ? __ldcg(gth + q) : 0u;
-      if ((tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= 8 && k <= 32 &&
-          (int)gridDim.x >= k && mine && q < nq) {
-        // Every CTA publishes its best score for the query.  The k-th best of
+      if (heads_turn(tile_i) && mine && q < nq) {
+        // Every CTA has published its best score for the query.  The k-th best of
         // the maxima of 32 groups of CTAs is reached by k vectors; with all
         // CTAs' rows behind it, few vectors of a tile reach it (a CTA's own
         // list is beaten by k / i vectors of its tile i).  It costs about 5 us, so
@@ -639,7 +642,6 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
           th_g = fmaxf(th_g, th_s);
           worst = 0;
           cnt = 0;
-          head = 0;
           th_s = -INFINITY;
           __syncwarp();
         }
@@ -725,10 +727,13 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       npark = 0;
       if (mine && q < nq && worst && th_s >= th_g) {  // a full list's k-th best
         const uint32_t b = order_bits(th_s);
-        if (b > published && b > shared_th) atomicMax(gth + q, b);
-        published = b;
+        if (b > shared_th) atomicMax(gth + q, b);
       }
-      if (mine && q < nq && head > head_out) heads[(size_t)blockIdx.x * nq + q] = head_out = head;
+      if (heads_turn(tile_i + 1) && mine && q < nq) {
+        uint64_t best = 0;
+        for (int i = 0; i < cnt; ++i) best = max(best, lst[i * MMA_M]);
+        heads[(size_t)blockIdx.x * nq + q] = (uint32_t)(best >> 32);
+      }
       asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
     }
     if (mine && q < nq) {

@@ -851,7 +851,8 @@ __global__ void k_allow_bits(const uint32_t* __restrict__ tenants, int64_t T, in
 }
 
 // Bit b of query q's block mask: filter block b holds a tenant the query
-// allows (its tenant bitmap shares a bit with the query's allow bitmap).  A
+// allows (its tenant bitmap shares a bit with the query's allow bitmap), for
+// filters whose bitmaps k_filter_prep has no shared memory for.  A
 // warp owns one mask word (32 blocks): lane w reads word w of each block's
 // bitmap, all 32 blocks' loads in flight at once.
 __global__ void __launch_bounds__(256)
@@ -877,6 +878,73 @@ k_block_mask(const uint32_t* __restrict__ block_bits, int64_t nblocks, int words
     for (int j = 0; j < 32; ++j) bits |= (__any_sync(FULL, x[j] != 0u) ? 1u : 0u) << j;
   }
   if (lane == 0) mask[q * mask_words + mw] = bits;
+}
+
+// The block masks (k_block_mask) and the allow bitmaps in one kernel: writes the
+// allow bitmap (as k_allow_bits; the first block of each query).
+// A warp owns one mask word (32 blocks, one per lane).  Short allowlists, the
+// usual case, are looked up by the warps themselves, and a lane reads one word
+// of its block's bitmap per allowed tenant instead of the whole bitmap (32
+// words with 1,000 tenants).  Nothing here depends on the query rotation, the
+// kernel before it, so it starts beside it (programmatic launch) and waits for
+// it only at its end, for the scan's sake.  One query, 100,000 rows, 1,000
+// tenants: whole search 46 -> 38 us.
+constexpr int ALLOW_SHORT = 32;  // tenants looked up by each warp; longer lists go through the bitmap
+__global__ void __launch_bounds__(256)
+k_filter_prep(const uint32_t* __restrict__ block_bits, int64_t nblocks, int words,
+              const uint32_t* __restrict__ tenants, int64_t T, const int64_t* __restrict__ off,
+              const uint32_t* __restrict__ ids, uint32_t* __restrict__ allow, int mask_words,
+              uint32_t* __restrict__ mask) {
+  extern __shared__ uint32_t bits_s[];  // the query's allow bitmap, long lists only
+  const int64_t q = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31;
+  griddep_launch_dependents();
+  const int64_t a = off[q], len = off[q + 1] - a;
+  const bool shrt = len <= ALLOW_SHORT;
+  uint32_t* out = allow + q * words;
+  int pos = -1;  // the lane's allowed tenant (short lists)
+  if (shrt) {
+    if (lane < len) pos = (int)find_tenant(tenants, T, ids[a + lane]);
+  } else {
+    for (int w = tid; w < words; w += blockDim.x) bits_s[w] = 0u;
+    __syncthreads();
+    for (int64_t j = tid; j < len; j += blockDim.x) {
+      const int64_t p = find_tenant(tenants, T, ids[a + j]);
+      if (p >= 0) atomicOr(bits_s + (p >> 5), 1u << (p & 31));
+    }
+    __syncthreads();
+  }
+  if (blockIdx.x == 0) {
+    if (shrt) {
+      for (int w0 = tid & ~31; w0 < words; w0 += blockDim.x) {  // whole warps
+        uint32_t x = 0;
+        for (int j = 0; j < (int)len; ++j) {
+          const int p = __shfl_sync(FULL, pos, j);
+          if (p >= 0 && (p >> 5) == w0 + lane) x |= 1u << (p & 31);
+        }
+        if (w0 + lane < words) out[w0 + lane] = x;
+      }
+    } else {
+      for (int w = tid; w < words; w += blockDim.x) out[w] = bits_s[w];
+    }
+  }
+  const int64_t mw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
+  if (mw < mask_words) {  // whole warps
+    const int64_t b = mw * 32 + lane;
+    const uint32_t* bb = block_bits + b * words;
+    bool hit = false;
+    if (shrt) {
+      for (int j = 0; j < (int)len; ++j) {
+        const int p = __shfl_sync(FULL, pos, j);
+        if (p >= 0 && b < nblocks) hit |= (__ldg(bb + (p >> 5)) >> (p & 31)) & 1u;
+      }
+    } else if (b < nblocks) {
+      for (int w = 0; w < words; ++w) hit |= (__ldg(bb + w) & bits_s[w]) != 0u;
+    }
+    const uint32_t word = __ballot_sync(FULL, hit);
+    if (lane == 0) mask[q * mask_words + mw] = word;
+  }
+  griddep_wait();  // the rotated queries are complete when this kernel is
 }
 
 // Rows v0 .. v0+n-1 get their dense tenant index and set their bit in their
@@ -1089,13 +1157,27 @@ cudaError_t launch_allow_bits(const FilterDev& f, const int64_t* allow_off,
   return cudaGetLastError();
 }
 
-cudaError_t launch_block_mask(const FilterDev& f, const uint32_t* allow, int64_t nq, uint32_t* mask,
+static cudaError_t launch_block_mask(const FilterDev& f, const uint32_t* allow, int64_t nq, uint32_t* mask,
                               cudaStream_t s) {
   if (nq == 0) return cudaSuccess;
   const int mw = filter_mask_words(f);
   const dim3 grid((unsigned)((mw + 7) / 8), (unsigned)nq);
   k_block_mask<<<grid, 256, 0, s>>>(f.block_bits, (f.n + f.block - 1) / f.block, f.words, allow, mw, mask);
   return cudaGetLastError();
+}
+
+cudaError_t launch_filter_prep(const FilterDev& f, const int64_t* allow_off, const uint32_t* allow_tenants,
+                               int64_t nq, uint32_t* allow, uint32_t* mask, cudaStream_t s) {
+  if (nq == 0) return cudaSuccess;
+  if ((size_t)f.words * sizeof(uint32_t) > 48 * 1024) {
+    const cudaError_t e = launch_allow_bits(f, allow_off, allow_tenants, nq, allow, s);
+    return e == cudaSuccess ? launch_block_mask(f, allow, nq, mask, s) : e;
+  }
+  const int mw = filter_mask_words(f);
+  const dim3 grid((unsigned)((mw + 7) / 8), (unsigned)nq);
+  return launch_maybe_pdl(s != nullptr, k_filter_prep, grid, dim3(256), (size_t)f.words * sizeof(uint32_t), s,
+                          (const uint32_t*)f.block_bits, (f.n + f.block - 1) / f.block, f.words,
+                          (const uint32_t*)f.tenants, f.n_tenants, allow_off, allow_tenants, allow, mw, mask);
 }
 
 cudaError_t launch_filter_build(const uint32_t* tenant_ids, FilterDev& f, cudaStream_t s) {

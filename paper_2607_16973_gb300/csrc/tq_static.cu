@@ -131,8 +131,7 @@ extern "C" tq_status tq_search_static(const float* Q, int64_t nq, int d, const f
   float* cand_s = reinterpret_cast<float*>(base + rot + allow + mask);
   int32_t* cand_i = reinterpret_cast<int32_t*>(base + rot + allow + mask + cs);
   e = tq::launch_rotate(Q, nq, d, R, qrot, status, counters, nq, s);
-  if (e == cudaSuccess && f) e = tq::launch_allow_bits(*f, allow_off, allow_tenants, nq, allow_bits, s);
-  if (e == cudaSuccess && f) e = tq::launch_block_mask(*f, allow_bits, nq, bmask, s);
+  if (e == cudaSuccess && f) e = tq::launch_filter_prep(*f, allow_off, allow_tenants, nq, allow_bits, bmask, s);
   if (e == cudaSuccess)
     e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, nullptr, f, allow_bits, bmask,
                             tq::search_path() == TQ_PATH_LUT_FIXED && d >= tq::kFixMinD, k, gx, cand_s, cand_i,
