@@ -48,7 +48,8 @@ SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_f
   const bool mma = mma_supported(bits, d, k);
   p.grid_mma = mma ? scan_mma_grid_x(nq, n, k, bits) : 0;
   p.grid_fold = fold_supported(bits, d, k, n) ? scan_fold_grid_x(nq, n) : 0;
-  const bool tm = scan_tm_supported(nq, n, d, bits, k, true), tm16 = scan_tm_supported(nq, n, d, bits, k, false);
+  const bool tm = scan_tm_supported(nq, n, d, bits, k, true, filter != nullptr);
+  const bool tm16 = scan_tm_supported(nq, n, d, bits, k, false, filter != nullptr);
   p.grid_tm = tm || tm16 ? scan_tm_grid_x(n) : 0;
   const int per_query = std::max(std::max(std::max(p.grid_lut, p.grid_mma), p.grid_fold) * k,
                                  p.grid_tm * scan_tm_list(k, tm));
@@ -490,9 +491,11 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
   // against 228 us per query at 999,000 x 1536)
   const bool use_fold = !use_mma && can_fold && path == TQ_PATH_LUT_FOLD;
   // AUTO: the small-batch tensor-core scan, exact (bounds, then float32
-  // scores) for unfiltered batches the lookup scan would take, fp16 above
-  const bool tm_bound = path == TQ_PATH_AUTO && !use_mma && !filter && tq::scan_tm_supported(nq, n, d, bits, k, true);
-  const bool use_tm = tm_bound || (path == TQ_PATH_AUTO && use_mma && tq::scan_tm_supported(nq, n, d, bits, k, false));
+  // scores) for batches the lookup scan would take, fp16 above
+  const bool filtered = filter != nullptr;
+  const bool tm_bound = path == TQ_PATH_AUTO && !use_mma && tq::scan_tm_supported(nq, n, d, bits, k, true, filtered);
+  const bool use_tm =
+      tm_bound || (path == TQ_PATH_AUTO && use_mma && tq::scan_tm_supported(nq, n, d, bits, k, false, filtered));
   const tq::SearchPlan p = tq::plan_search(nq, n, d, bits, k, filter);
   if (ws_bytes < p.total)
     return fail(TQ_EINVAL, "tq_search: workspace of %zu bytes, %zu needed", ws_bytes, p.total);
@@ -516,18 +519,22 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
   if (use_tm) {
     float* lows = reinterpret_cast<float*>(ws + p.off_lows);
     int* gate = reinterpret_cast<int*>(ws + p.off_gate);
-    if (e == cudaSuccess && filter) e = tq::launch_allow_bits(filter->f, allow_off, allow_tenants, nq, allow, s);
+    if (e == cudaSuccess && filter)
+      e = tm_bound ? tq::launch_filter_prep(filter->f, allow_off, allow_tenants, nq, allow, bmask, s)
+                   : tq::launch_allow_bits(filter->f, allow_off, allow_tenants, nq, allow, s);
     if (e == cudaSuccess)
       e = tq::launch_scan_tm(qrot, nq, d, centroids, codes, scale, n, deleted, filter ? filter->f.dense : nullptr,
-                             allow, filter ? filter->f.words : 0, bias, k, tm_bound, cs, ci, status, force, gth, lows, s,
+                             allow, filter ? filter->f.words : 0, tm_bound ? bmask : nullptr,
+                             filter ? tq::filter_mask_words(filter->f) : 0, filter ? filter->f.block : 64, bias, k,
+                             tm_bound, cs, ci, status, force, gth, lows, s,
                              (cudaEvent_t)tq::profile_start(), (cudaEvent_t)tq::profile_stop());
     if (tm_bound) {
       if (e == cudaSuccess)
         e = tq::launch_rescore(qrot, nq, d, centroids, codes, scale, n, k, cs, ci, lows, force, gate, ext_ids, out_ids,
                                out_scores, bias, s);
       if (e == cudaSuccess)
-        e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, deleted, nullptr, nullptr, nullptr,
-                                false, k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias,
+        e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
+                                filter ? &filter->f : nullptr, allow, bmask, false, k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias,
                                 gate, s, nullptr, nullptr);
     } else if (e == cudaSuccess) {
       e = tq::launch_merge(cs, ci, nq, p.grid_tm * k, k, ext_ids, out_ids, out_scores, s);

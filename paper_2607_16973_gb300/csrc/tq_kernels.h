@@ -155,13 +155,14 @@ cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* c
 // for values the bounds do not cover (both zeroed by the query rotation); lows [2][nq][grid_x] are lower bounds of
 // each list's best and k-th best score.
 // Without it, fp16 scores of at most 32 queries: lists of k for launch_merge.
-bool scan_tm_supported(int64_t nq, int64_t n, int d, int bits, int k, bool bound);
+// `bmask` (nullable, bound only): the block masks of launch_filter_prep.
+bool scan_tm_supported(int64_t nq, int64_t n, int d, int bits, int k, bool bound, bool filtered);
 int scan_tm_list(int k, bool bound);
 int scan_tm_grid_x(int64_t n);
 cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* centroids, const uint8_t* codes,
                            const float* scale, int64_t n, const uint32_t* del, const uint32_t* dense,
-                           const uint32_t* allow_bits, int words, const float* bias, int k, bool bound, float* cand_s,
-                           int32_t* cand_i, int* err, int* force, uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
+                           const uint32_t* allow_bits, int words, const uint32_t* bmask, int mask_words, int fblock,
+                           const float* bias, int k, bool bound, float* cand_s, int32_t* cand_i, int* err, int* force, uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
                            cudaEvent_t ev1);
 cudaError_t launch_rescore(const float* qrot, int64_t nq, int d, const float* centroids, const uint8_t* codes,
                            const float* scale, int64_t n, int k, const float* cand_s, const int32_t* cand_i,

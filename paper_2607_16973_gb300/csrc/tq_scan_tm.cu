@@ -71,6 +71,8 @@ constexpr uint32_t TM_SMEM_MAX = 232448;  // 227 KB per block
 // The upper half of each 256-byte table row is free (a byte permute makes the
 // entry's address only with that row size): 8,192 words, of which 2 * N * 128
 // hold two tiles' candidate scores (and with 16 columns 2 * 128 their |scale|).
+constexpr int TM_TILE_LIST = 2 * 16 * TM_M + 2 * TM_M;  // first word of the tile list (16 columns)
+constexpr int TM_MAX_TILES = 8192 - TM_TILE_LIST;
 constexpr int TM_LIST = 32;               // entries of a query's list in a CTA (one per lane)
 constexpr uint32_t TM_A_COL = 128;        // TMEM: two sets of two accumulators of N <= 32 columns, then the stages
 // misc area (after the raw tiles): per-query values, masks, barriers
@@ -80,7 +82,8 @@ struct TmMisc {
   static constexpr uint32_t bars = 1536;                              // 35 mbarriers
   static constexpr uint32_t slot = bars + 36 * 8;                     // TMEM address, abort flag
   static constexpr uint32_t any = slot + 16;                          // uint32 [2][4]: queries with a candidate, by warp
-  static constexpr uint32_t total = any + 32;
+  static constexpr uint32_t tiles = any + 32;                         // int: tiles in the list
+  static constexpr uint32_t total = tiles + 4;
 };
 static_assert(TmMisc::total <= 2048, "misc area");
 
@@ -213,7 +216,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
 k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict__ qrot,
           const float* __restrict__ centroids, const float* __restrict__ scale, const uint32_t* __restrict__ del,
           const uint32_t* __restrict__ dense, const uint32_t* __restrict__ allow_bits, int words,
-          const float* __restrict__ bias, int n, int nq, int d, int k, int C, int cst, float* __restrict__ cand_s,
+          const uint32_t* __restrict__ bmask, int mask_words, int fblock, const float* __restrict__ bias, int n, int nq, int d, int k, int C, int cst, float* __restrict__ cand_s,
           int* __restrict__ cand_i, int* __restrict__ err, int* __restrict__ force, uint32_t* __restrict__ gth,
           float* __restrict__ lows) {
   extern __shared__ unsigned char smem_dyn[];
@@ -242,10 +245,18 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
 
   const int tid = threadIdx.x, warp = __shfl_sync(FULL, tid >> 5, 0), lane = tid & 31;
   const int ntiles = (n + TM_M - 1) / TM_M;
-  const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int all_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int raws = d >> 8;        // raw code tiles per vector tile
   const int blks = d / TM_BLK;    // decoded blocks per vector tile
-  const int total_ld = my_tiles * raws, total_it = my_tiles * blks;
+  // With block masks (BOUND searches with a filter) the CTA walks the tiles
+  // that hold a filter block some query allows (Sec. III-B: skipped before any
+  // code byte is read), listed behind the candidate slots.
+  int my_tiles = all_tiles;
+  int* s_tiles = reinterpret_cast<int*>(misc + TmMisc::tiles);
+  auto tile_at = [&](int i) {
+    return BOUND && bmask ? *reinterpret_cast<const int*>(gapw(TM_TILE_LIST + i))
+                          : (int)blockIdx.x + i * (int)gridDim.x;
+  };
 
   griddep_launch_dependents();
   if (tid == 0) {
@@ -276,13 +287,13 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
 
   auto issue = [&](int ld) {
     const int s = ld % cst;
-    const int t = (int)blockIdx.x + (ld / raws) * (int)gridDim.x;
+    const int t = tile_at(ld / raws);
     mbar_arrive_expect_tx(cfull + s, TM_RAW);
     tma_load_2d(sRaw + (size_t)s * TM_RAW, &codes_map, (ld % raws) * 128, t * TM_M, cfull + s);
   };
   int issued = 0;
-  if (warp == TM_PROD && lane == 0)  // the first code tiles go out before the tables are built
-    for (; issued < cst && issued < total_ld; ++issued) issue(issued);
+  if (warp == TM_PROD && lane == 0 && !bmask)  // the first code tiles go out before the tables are built
+    for (; issued < cst && issued < all_tiles * raws; ++issued) issue(issued);
 
   // the codebook in fp16: BOUND scales it by a power of two to [1, 2) at its
   // largest centroid and takes the largest rounding error
@@ -307,7 +318,19 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
     *reinterpret_cast<uint4*>(lut + x * 256 + (i & 7) * 16) = make_uint4(v, v, v, v);
   }
   for (int i = tid; i < 2 * N * 4; i += TM_THREADS) s_mask[i] = 0u;
+  if (tid == 0) *s_tiles = 0;
+  if (BOUND && bmask) __syncthreads();
   griddep_wait();  // the rotated queries (and allow bitmaps, TQ+ terms) are written
+  if (BOUND && bmask) {
+    const int per = TM_M / fblock;  // 2 or 4 filter blocks a tile, in one mask word
+    for (int i = tid; i < all_tiles; i += TM_THREADS) {
+      const int t = (int)blockIdx.x + i * (int)gridDim.x, b = t * per;
+      uint32_t any = 0;
+      for (int q = 0; q < nq; ++q) any |= __ldg(bmask + (size_t)q * mask_words + (b >> 5));
+      if ((any >> (b & 31)) & ((1u << per) - 1u))
+        *reinterpret_cast<int*>(gapw(TM_TILE_LIST + atomicAdd(s_tiles, 1))) = t;
+    }
+  }
   // The query block: a warp per column, d fp16 values, K-major with the
   // 128-byte swizzle in blocks of 64 coordinates; columns past nq are zero.
   for (int q = warp; q < N; q += TM_THREADS / 32) {
@@ -381,13 +404,15 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (BOUND && bmask) my_tiles = *s_tiles;
+  const int total_ld = my_tiles * raws, total_it = my_tiles * blks;
 
   if (warp == TM_PROD) {
     // ------------------------------------------------- code tiles (TMA, HBM)
     if (lane == 0) {
       for (; issued < total_ld; ++issued) {
         const int s = issued % cst, use = issued / cst;
-        if (!mbar_wait(cempty + s, (use - 1) & 1, abort_flag, err, 61)) break;
+        if (use > 0 && !mbar_wait(cempty + s, (use - 1) & 1, abort_flag, err, 61)) break;
         issue(issued);
       }
       // never leave with copies in flight: wait (bounded) for the last one of each stage
@@ -508,14 +533,14 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
     float sc_next = 0.f;
     uint32_t tn_next = 0;
     auto fetch = [&](int tile_i) {
-      const int v = ((int)blockIdx.x + tile_i * (int)gridDim.x) * TM_M + row;
-      const bool in = tile_i < my_tiles && v < n;
+      const int v = tile_i < my_tiles ? tile_at(tile_i) * TM_M + row : n;
+      const bool in = v < n;
       sc_next = in ? (scale ? __ldg(scale + v) : 1.0f) : 0.f;
       tn_next = in && allow_bits ? __ldg(dense + v) : 0u;
     };
     fetch(grp);
     for (int tile_i = grp; tile_i < my_tiles; tile_i += 2) {
-      const int t = (int)blockIdx.x + tile_i * (int)gridDim.x;
+      const int t = tile_at(tile_i);
       const int v = t * TM_M + row;
       const bool valid = v < n;
       const float sc = sc_next, asc = fabsf(sc);
@@ -859,8 +884,14 @@ k_rescore(const float* __restrict__ qrot, int d, const float* __restrict__ centr
 // The fp16 scan is faster than the batched one (which makes each CTA decode
 // 256-vector tiles and stream its queries) at every size: 16 queries 2,048 rows
 // 46 / 120, 100,000 67 / 187.
-bool scan_tm_supported(int64_t nq, int64_t n, int d, int bits, int k, bool bound) {
+// With a filter a tile is read when any query allows one of its blocks, so one
+// query, whose lookup scan skips 32-row steps, stays there; from two on the
+// tiles are read once for all of them.
+bool scan_tm_supported(int64_t nq, int64_t n, int d, int bits, int k, bool bound, bool filtered) {
   if (bits != 4 || d % 256 != 0 || d > 2048 || k > TM_LIST || nq < 1) return false;
+  if (filtered && bound)
+    return nq >= 2 && nq <= 16 && n * d * nq >= (int64_t)1 << 26 &&
+           (n + TM_M - 1) / TM_M <= (int64_t)TM_MAX_TILES * device_sm_count();
   if (bound) return nq <= 16 && n >= kTmMinRows && n * d * nq >= (k <= 16 ? (int64_t)1 << 24 : (int64_t)1 << 27);
   return nq <= 32;
 }
@@ -873,8 +904,8 @@ int scan_tm_grid_x(int64_t n) {
 
 cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* centroids, const uint8_t* codes,
                            const float* scale, int64_t n, const uint32_t* del, const uint32_t* dense,
-                           const uint32_t* allow_bits, int words, const float* bias, int k, bool bound, float* cand_s,
-                           int32_t* cand_i, int* err, int* force, uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
+                           const uint32_t* allow_bits, int words, const uint32_t* bmask, int mask_words, int fblock,
+                           const float* bias, int k, bool bound, float* cand_s, int32_t* cand_i, int* err, int* force, uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
                            cudaEvent_t ev1) {
   if (nq == 0) return cudaSuccess;
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
@@ -900,7 +931,7 @@ cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* ce
     const cudaError_t r = set_max_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)smem);
     if (r != cudaSuccess) return r;
     return launch_maybe_pdl(pdl, kernel, grid, block, smem, s, map, qrot, centroids, scale, del, dense, allow_bits,
-                            words, bias, (int)n, (int)nq, d, k, C, cst, cand_s, cand_i, err, force, gth, lows);
+                            words, bmask, mask_words, fblock, bias, (int)n, (int)nq, d, k, C, cst, cand_s, cand_i, err, force, gth, lows);
   };
   e = bound ? go(k_scan_tm<16, true>) : N == 16 ? go(k_scan_tm<16, false>) : go(k_scan_tm<32, false>);
   if (e != cudaSuccess) return e;

@@ -170,3 +170,31 @@ def test_fp16_batch_filtered(cuda_lib, tdev):
     allowed = np.stack([np.isin(tenants, ids_allowed[off[i]:off[i + 1]]) for i in range(nq)])
     ref = O.search(Q, R, c32, 4, packed, scale, k, d, tenant_ids=tenants, allow_off=off, allow_ids=ids_allowed)
     check_topk(ids, sc, ref.ids, ref.scores64, allowed, k, TOL_MMA)
+
+
+@pytest.mark.parametrize("order", ["interleaved", "sorted"])
+@pytest.mark.parametrize("block", [32, 64])
+def test_exact_search_filtered(cuda_lib, tdev, order, block):
+    """Tiles no query allows are passed over; lists of one tenant, of five, of
+    more than a warp looks up, with ids the corpus does not have, and empty."""
+    torch, T = tdev
+    tq = cuda_lib
+    d, n, nq, k = 512, 60_001, 6, 10
+    packed, scale, R, Q = _data(n, d, nq, seed=41)
+    c32, _ = _cb(d)
+    tenants, values = synth.zipf_tenants(n, 100)
+    if order == "sorted":
+        tenants = np.sort(tenants)
+    lists = [values[:1], values[50:55], values[10:43], values[60:92], np.append(values[99:], [5, 7]).astype(np.uint32),
+             values[:0]]
+    off = np.cumsum([0] + [len(v) for v in lists]).astype(np.int64)
+    ten = np.concatenate(lists).astype(np.uint32)
+    flt = tq.Filter(T(tenants.view(np.int32)), block=block)
+    a = (T(Q), T(R), T(c32), 4, T(packed), T(scale), k)
+    kw = dict(filter=flt, allow_off=T(off), allow_tenants=T(ten.view(np.int32)))
+    ids, sc = _search(tq, torch, "auto", *a, **kw)
+    ids_l, sc_l = _search(tq, torch, "lut", *a, **kw)
+    assert np.array_equal(ids, ids_l) and np.array_equal(sc, sc_l)
+    allowed = np.stack([np.isin(tenants, v) for v in lists])
+    ref = O.search(Q, R, c32, 4, packed, scale, k, d, tenant_ids=tenants, allow_off=off, allow_ids=ten)
+    check_topk(ids, sc, ref.ids, ref.scores64, allowed, k, TOL_LUT)
