@@ -43,6 +43,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "tq_internal.h"
 #include "tq_kernels.h"
@@ -67,7 +68,8 @@ constexpr size_t kPlanHead = 256;           // the plan: status word, then R_hi,
 struct HSmem {
   static constexpr uint32_t bnd = H_STAGES * H_STAGE_BYTES;  // [512] floats (one copy per bank up to 4 bits)
   static constexpr uint32_t cen = bnd + 512 * 4;             // [512] floats
-  static constexpr uint32_t part = cen + 512 * 4;            // [2][128] double: the second column half's sums
+  static constexpr uint32_t cell = cen + 512 * 4;            // [2048] (boundary, code below it) by cell
+  static constexpr uint32_t part = cell + 2048 * 8;          // [2][128] double: the second column half's sums
   static constexpr uint32_t bars = part + 2 * HM * 8;        // 19 mbarriers
   static constexpr uint32_t misc = bars + 20 * 8;            // TMEM address, abort flag, last flag
   static constexpr uint32_t total = misc + 16;
@@ -200,6 +202,7 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
   unsigned char* base = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
   float* sBnd = reinterpret_cast<float*>(base + HSmem::bnd);
   float* sCen = reinterpret_cast<float*>(base + HSmem::cen);
+  float2* sCell = reinterpret_cast<float2*>(base + HSmem::cell);
   double* sPart = reinterpret_cast<double*>(base + HSmem::part);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + HSmem::bars);
   uint64_t* full = bars;             // [4] X and R tiles landed
@@ -227,6 +230,32 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
     sCen[i] = e < L ? centroids[e] : 0.f;
     sBnd[i] = e < L - 1 ? boundaries[e] : INFINITY;
   }
+  // The code of z by cells: the boundaries' range is cut into MC equal cells, few
+  // enough apart that a cell holds at most one boundary; then the code is the
+  // count of boundaries in lower cells plus a comparison with the cell's own.
+  // One lookup instead of a search of BITS dependent ones, with the same
+  // result for every z (the cell is a monotone function of z, evaluated alike
+  // for z and the boundaries).  Where a cell would hold two (or the range is not
+  // finite), the search stays.
+  constexpr int MC = BITS <= 4 ? 128 : 2048;           // cells
+  constexpr int CREP = BITS <= 4 ? 16 : 1;             // copies (8-byte lookups: one per bank pair)
+  const float lo_b = __ldg(boundaries), hi_b = __ldg(boundaries + L - 2);
+  const float cs = (float)(MC - 3) / (hi_b - lo_b), co = 1.0f - lo_b * cs;
+  auto cell_of = [&](float z) {
+    const float f = fminf(fmaxf(fmaf(z, cs, co), 0.f), (float)(MC - 1));  // (NaN: 0)
+    return __float_as_int(f + 8388608.0f) & 0xFFFF;                      // rounded to the nearest
+  };
+  bool cells_ok = hi_b > lo_b && cs < 0x1p60f && fabsf(co) < 0x1p60f;
+  for (int i = tid; i < L; i += H_THREADS) {  // cells above the boundary before, up to boundary i's
+    const int prev = i == 0 ? -1 : cell_of(__ldg(boundaries + i - 1));
+    const float b = i < L - 1 ? __ldg(boundaries + i) : INFINITY;
+    const int c = i < L - 1 ? cell_of(b) : MC - 1;
+    if (i < L - 1 && c <= prev) cells_ok = false;
+    for (int j = prev + 1; j <= c; ++j)
+      for (int r = 0; r < CREP; ++r)
+        sCell[j * CREP + r] = make_float2(j == c && i < L - 1 ? b : INFINITY, __int_as_float(i));
+  }
+  cells_ok = __syncthreads_and(cells_ok);
   if (tid == 0) {
     for (int s = 0; s < H_STAGES; ++s) {
       mbar_init(full + s, 1);
@@ -380,7 +409,8 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
     double c2 = 0.0, yc = 0.0;  // the row's sums over this thread's columns (float per 16, then double)
     int64_t grow = 0;
     // 16 consecutive accumulator columns (coordinates j0 .. j0+15) of this row
-    auto group = [&](const uint32_t (&r)[16], int j0) {
+    const float2* my_cell = sCell + (lane & (CREP - 1));
+    auto group = [&](const uint32_t (&r)[16], int j0, auto by_cell) {
       if (j0 >= d) return;  // columns of a partial last chunk (d is a multiple of 32)
       uint64_t packed = 0;  // 2-, 3- and 4-bit codes, little-endian bit stream
       uint32_t p8[4] = {0, 0, 0, 0};
@@ -400,9 +430,14 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
             z = (y - mu) * (1.0f / a);
           }
           int code = 0;
+          if constexpr (decltype(by_cell)::value) {
+            const float2 e = my_cell[cell_of(z) * CREP];
+            code = __float_as_int(e.y) + (z > e.x ? 1 : 0);
+          } else {
 #pragma unroll
-          for (int step = L / 2; step >= 1; step >>= 1)
-            if (z > sBnd[(code + step - 1) * REP + rl]) code += step;
+            for (int step = L / 2; step >= 1; step >>= 1)
+              if (z > sBnd[(code + step - 1) * REP + rl]) code += step;
+          }
           const float cc = sCen[code * REP + rl];
           const float cv = CAL ? fmaf(a, cc, mu) : cc;
           g2 = fmaf(cv, cv, g2);
@@ -444,18 +479,22 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
       if (!warp_wait(acc_full, (uint32_t)(cs & 1), abort_flag, err, 75)) break;
       tc_fence_after();
       const int jb = c * N + h * (N / 2);
-      uint32_t ra[16], rb[16];
-      tmem_ld16_issue(tl, ra);
-      tmem_wait16(ra);
+      auto read_out = [&](auto by_cell) {
+        uint32_t ra[16], rb[16];
+        tmem_ld16_issue(tl, ra);
+        tmem_wait16(ra);
 #pragma unroll 1
-      for (int g = 0; g < N / 2; g += 32) {
-        tmem_ld16_issue(tl + (uint32_t)(g + 16), rb);
-        group(ra, jb + g);
-        tmem_wait16(rb);
-        if (g + 32 < N / 2) tmem_ld16_issue(tl + (uint32_t)(g + 32), ra);
-        group(rb, jb + g + 16);
-        if (g + 32 < N / 2) tmem_wait16(ra);
-      }
+        for (int g = 0; g < N / 2; g += 32) {
+          tmem_ld16_issue(tl + (uint32_t)(g + 16), rb);
+          group(ra, jb + g, by_cell);
+          tmem_wait16(rb);
+          if (g + 32 < N / 2) tmem_ld16_issue(tl + (uint32_t)(g + 32), ra);
+          group(rb, jb + g + 16, by_cell);
+          if (g + 32 < N / 2) tmem_wait16(ra);
+        }
+      };
+      if (cells_ok) read_out(std::true_type{});
+      else read_out(std::false_type{});
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty);
