@@ -14,13 +14,15 @@
 // undone exactly.
 //
 // What bounds it: 3 * 2 d^2 fp16 flops per row (14.1 TFLOP for 999,000 x 1536:
-// 7.3 ms at 1,936 TFLOP/s); on top come the accumulator's read-out between
-// chunks (tensor memory holds one accumulator of 256 columns beside the split
-// X tiles), the split itself, which 8 warps just keep up with, and the norms'
-// pass over X (0.95 ms).  Measured at 999,000 x 1536, 4-bit: 20.1 ms (TF32) ->
-// 12.8 ms; 1,000 rows 375 -> 47 us; 40,003 x 768 at 8 bits 444 -> 320 us.  Four
-// converter groups (72 registers, the epilogue spills) 13.9 ms; separate rings
-// of 3 X and 5 R stages 13.7 ms.
+// 7.3 ms at 1,936 TFLOP/s), under the power cap at that rate (the SM clock falls
+// to 1.65-1.95 GHz); with the loads, the split and the read-out taken out the
+// kernel takes 7.1 ms and the norms' pass over X 0.95.  On top come X's way to
+// the SMs, once per chunk (about 2 ms), its split, which 8 warps just keep up
+// with (2.4 ms), and R's tiles (1 ms).  Measured at 999,000 x 1536, 4-bit: 20.1 ms
+// (TF32) -> 12.1 ms; 1,000 rows 375 -> 48 us; 40,003 x 768 at 8 bits 444 -> 184 us.
+// Two accumulators of 192 columns hide the read-out behind the next chunk; with
+// one of 256 it took 12.7 ms and 211 us.  Four converter groups (72 registers,
+// the epilogue spills) 14.0 ms; separate rings of 3 X and 5 R stages 13.7 ms.
 //
 // Work.  The items are (128-row panel, chunk of N output coordinates), panel by
 // panel; each CTA takes an equal run of items, so the SMs finish together
@@ -30,7 +32,7 @@
 // Per K-block a stage holds the raw X tile (128 x 32 fp32, 128-byte swizzle) and
 // the R_hi, R_lo tiles (N x 32 fp16, 64-byte swizzle); the split X goes to
 // tensor memory (A operand).  K-blocks are walked alternately forwards and
-// backwards, by the 256-coordinate block a chunk lies in, so that a chunk
+// backwards, by the 192-coordinate block a chunk lies in, so that a chunk
 // starts on the X tiles the previous one read last, and an output coordinate's
 // sum does not depend on N.  Roles (18 warps): 0-7 converters (two groups of
 // four, alternate K-blocks), 8 producer, 9 MMA issuer, 10-17 epilogue (lane
@@ -55,14 +57,14 @@ namespace {
 
 constexpr int HM = 128;                     // rows of X per panel (MMA M)
 constexpr int HK = 32;                      // coordinates per K-block
-constexpr int H_MAXN = 256;                 // output coordinates per chunk (MMA N), at most
+constexpr int H_MAXN = 192;                 // output coordinates per chunk (MMA N): 192, 96 or 64
 constexpr int H_STAGES = 4;
 constexpr int HX_BYTES = HM * HK * 4;       // 16 KB
-constexpr int HR_BYTES = H_MAXN * HK * 2;   // 16 KB: room for an R_hi or R_lo tile
+constexpr int HR_BYTES = H_MAXN * HK * 2;   // 12 KB: room for an R_hi or R_lo tile
 constexpr int H_STAGE_BYTES = HX_BYTES + 2 * HR_BYTES;
 constexpr int H_CONV = 8, H_PROD = 8, H_MMA = 9, H_EPI0 = 10, H_EPI = 8;
 constexpr int H_THREADS = (H_EPI0 + H_EPI) * 32;  // 576
-constexpr uint32_t H_TM_A = 256;            // TMEM column of the first stage's x_hi (16 columns), then x_lo
+constexpr uint32_t H_TM_A = 2 * H_MAXN;     // TMEM: two accumulators, then per stage x_hi (16 columns) and x_lo
 constexpr size_t kPlanHead = 256;           // the plan: status word, then R_hi, R_lo in fp32 (tq_encode_tc.cu)
 
 struct HSmem {
@@ -70,8 +72,8 @@ struct HSmem {
   static constexpr uint32_t cen = bnd + 512 * 4;             // [512] floats
   static constexpr uint32_t cell = cen + 512 * 4;            // [2048] (boundary, code below it) by cell
   static constexpr uint32_t part = cell + 2048 * 8;          // [2][128] double: the second column half's sums
-  static constexpr uint32_t bars = part + 2 * HM * 8;        // 19 mbarriers
-  static constexpr uint32_t misc = bars + 20 * 8;            // TMEM address, abort flag, last flag
+  static constexpr uint32_t bars = part + 2 * HM * 8;        // 21 mbarriers
+  static constexpr uint32_t misc = bars + 22 * 8;            // TMEM address, abort flag, last flag
   static constexpr uint32_t total = misc + 16;
 };
 constexpr uint32_t kHSmem = HSmem::total + 1024;
@@ -208,8 +210,8 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
   uint64_t* full = bars;             // [4] X and R tiles landed
   uint64_t* conv = bars + 4;         // [4] X tile split into tensor memory
   uint64_t* empty = bars + 8;        // [4] MMAs done with the stage
-  uint64_t* acc_full = bars + 12;    // the accumulator complete
-  uint64_t* acc_empty = bars + 13;   // the accumulator read out
+  uint64_t* acc_full = bars + 12;    // [2] accumulator complete
+  uint64_t* acc_empty = bars + 19;   // [2] accumulator read out
   uint64_t* part_ready = bars + 14;  // the second column half's row sums of a panel written
   uint64_t* part_free = bars + 15;   // and read
   uint64_t* fin = bars + 16;
@@ -262,8 +264,10 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
       mbar_init(conv + s, 4);
       mbar_init(empty + s, 1);
     }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, H_EPI);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(acc_full + s, 1);
+      mbar_init(acc_empty + s, H_EPI);
+    }
     mbar_init(part_ready, HM);
     mbar_init(part_free, 4);
     mbar_init(fin, 1);
@@ -289,7 +293,7 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
       bool ok = true;
       for (int64_t item = i0; item < i1 && ok; ++item) {
         const int panel = (int)(item / C), c = (int)(item % C);
-        const bool back = ((c * N) >> 8) & 1;
+        const bool back = (c * N / H_MAXN) & 1;
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = (int)(it % H_STAGES);
           const int64_t use = it / H_STAGES;
@@ -319,7 +323,9 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
     int s = 0, par = 0;
     bool ok = true;
     for (int64_t cs = 0; cs < chunks && ok; ++cs) {
-      if (cs >= 1 && !warp_wait(acc_empty, (uint32_t)((cs - 1) & 1), abort_flag, err, 72)) break;
+      const int set = (int)(cs & 1);
+      const uint32_t dt = tm + (uint32_t)(set * H_MAXN);
+      if (cs >= 2 && !warp_wait(acc_empty + set, (uint32_t)(((cs >> 1) - 1) & 1), abort_flag, err, 72)) break;
       for (int kb = 0; kb < KB; ++kb) {
         if (!warp_wait(conv + s, (uint32_t)par, abort_flag, err, 73)) {
           ok = false;
@@ -332,12 +338,12 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
         if (h_elect()) {
 #pragma unroll
           for (int kk = 0; kk < HK / 16; ++kk) {  // 16 values: 32 bytes of each R row, 8 TMEM columns of x
-            h_mma(tm, ah + kk * 8u, rh + kk * 2u, idesc, kk ? 1u : more);
-            h_mma(tm, ah + kk * 8u, rl + kk * 2u, idesc, 1u);
-            h_mma(tm, al + kk * 8u, rh + kk * 2u, idesc, 1u);
+            h_mma(dt, ah + kk * 8u, rh + kk * 2u, idesc, kk ? 1u : more);
+            h_mma(dt, ah + kk * 8u, rl + kk * 2u, idesc, 1u);
+            h_mma(dt, al + kk * 8u, rh + kk * 2u, idesc, 1u);
           }
           mma_commit(empty + s);
-          if (kb == KB - 1) mma_commit(acc_full);
+          if (kb == KB - 1) mma_commit(acc_full + set);
         }
         __syncwarp();
         if (++s == H_STAGES) {
@@ -476,28 +482,33 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
         c2 = 0.0;
         yc = 0.0;
       }
-      if (!warp_wait(acc_full, (uint32_t)(cs & 1), abort_flag, err, 75)) break;
+      const int set = (int)(cs & 1);
+      if (!warp_wait(acc_full + set, (uint32_t)((cs >> 1) & 1), abort_flag, err, 75)) break;
       tc_fence_after();
       const int jb = c * N + h * (N / 2);
+      const uint32_t ts = tl + (uint32_t)(set * H_MAXN);
+      const int G16 = N / 32;  // 16-column groups of this half
       auto read_out = [&](auto by_cell) {
         uint32_t ra[16], rb[16];
-        tmem_ld16_issue(tl, ra);
+        tmem_ld16_issue(ts, ra);
         tmem_wait16(ra);
 #pragma unroll 1
-        for (int g = 0; g < N / 2; g += 32) {
-          tmem_ld16_issue(tl + (uint32_t)(g + 16), rb);
-          group(ra, jb + g, by_cell);
+        for (int g = 0; g < G16; g += 2) {
+          const bool two = g + 1 < G16, more = g + 2 < G16;
+          if (two) tmem_ld16_issue(ts + (uint32_t)(16 * g + 16), rb);
+          group(ra, jb + 16 * g, by_cell);
+          if (!two) break;
           tmem_wait16(rb);
-          if (g + 32 < N / 2) tmem_ld16_issue(tl + (uint32_t)(g + 32), ra);
-          group(rb, jb + g + 16, by_cell);
-          if (g + 32 < N / 2) tmem_wait16(ra);
+          if (more) tmem_ld16_issue(ts + (uint32_t)(16 * g + 32), ra);
+          group(rb, jb + 16 * g + 16, by_cell);
+          if (more) tmem_wait16(ra);
         }
       };
       if (cells_ok) read_out(std::true_type{});
       else read_out(std::false_type{});
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty);
+      if (lane == 0) mbar_arrive(acc_empty + set);
       if (c != C - 1 && item != i1 - 1) continue;
       // the panel's scalar (step 5), or this CTA's part of it: the second
       // column half hands its sums to the first, row by row
@@ -574,14 +585,14 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
 // Output coordinates per chunk: the N that the fewest cycles are expected of.
 // A K-block takes as long as its MMAs (3 N cycles), its tiles' way from L2
 // (16 KB of X and 128 N bytes of R at about 55 bytes per cycle) or its
-// conversion (about 300); an SM takes ceil(items / SMs) of them in turn.
+// conversion (about 350); an SM takes ceil(items / SMs) of them in turn.
 int encode_h_chunk(int64_t n, int d) {
   const int64_t panels = (n + HM - 1) / HM, sms = device_sm_count();
   int best = H_MAXN;
   double best_t = 1e300;
-  for (int N = H_MAXN; N >= 64; N >>= 1) {
+  for (const int N : {192, 96, 64}) {
     const int64_t items = panels * ((d + N - 1) / N);
-    const double kb = std::max({300.0, 3.0 * N, (16384.0 + 128.0 * N) / 55.0});
+    const double kb = std::max({350.0, 3.0 * N, (16384.0 + 128.0 * N) / 55.0});
     const double t = (double)((items + sms - 1) / sms) * kb;
     if (t < best_t) {
       best_t = t;
