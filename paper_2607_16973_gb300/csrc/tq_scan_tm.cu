@@ -15,7 +15,9 @@
 // register decode costs about 21 integer instructions per 8 codes, at 64 lanes
 // per cycle and SM.  The query block of the whole contraction stays in shared
 // memory for the kernel's life (N x d fp16), so no query bytes are re-read per
-// tile.  Measured at 999,000 x 1536, whole searches: one query, top-5, 217 us
+// tile.  (Decoding a quarter of the words with byte permutes instead of lookups,
+// to relieve that datapath, was slower, 185 us against 170: with 27 warps the
+// decoders are as close to the issue rate.)  Measured at 999,000 x 1536, whole searches: one query, top-5, 217 us
 // (lookup scan) -> 165; 32 queries 484 us (k_scan_mma) -> 216; eight queries
 // over 250,007 rows 425 us -> 115.
 //
@@ -211,7 +213,7 @@ __device__ __noinline__ uint64_t list_add(uint64_t list, uint64_t cand, uint32_t
   return list_merge(list, __shfl_sync(FULL, cand, 31 - lane));
 }
 
-template <int N, bool BOUND>
+template <int N, bool BOUND, bool MASKED>
 __global__ void __launch_bounds__(TM_THREADS, 1)
 k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict__ qrot,
           const float* __restrict__ centroids, const float* __restrict__ scale, const uint32_t* __restrict__ del,
@@ -248,13 +250,13 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
   const int all_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int raws = d >> 8;        // raw code tiles per vector tile
   const int blks = d / TM_BLK;    // decoded blocks per vector tile
-  // With block masks (BOUND searches with a filter) the CTA walks the tiles
+  // With block masks (MASKED: BOUND searches with a filter) the CTA walks the tiles
   // that hold a filter block some query allows (Sec. III-B: skipped before any
   // code byte is read), listed behind the candidate slots.
-  int my_tiles = all_tiles;
+  int my_tiles = all_tiles;  // (MASKED: set when the list is complete)
   int* s_tiles = reinterpret_cast<int*>(misc + TmMisc::tiles);
   auto tile_at = [&](int i) {
-    return BOUND && bmask ? *reinterpret_cast<const int*>(gapw(TM_TILE_LIST + i))
+    return MASKED ? *reinterpret_cast<const int*>(gapw(TM_TILE_LIST + i))
                           : (int)blockIdx.x + i * (int)gridDim.x;
   };
 
@@ -292,7 +294,7 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
     tma_load_2d(sRaw + (size_t)s * TM_RAW, &codes_map, (ld % raws) * 128, t * TM_M, cfull + s);
   };
   int issued = 0;
-  if (warp == TM_PROD && lane == 0 && !bmask)  // the first code tiles go out before the tables are built
+  if (warp == TM_PROD && lane == 0 && !MASKED)  // the first code tiles go out before the tables are built
     for (; issued < cst && issued < all_tiles * raws; ++issued) issue(issued);
 
   // the codebook in fp16: BOUND scales it by a power of two to [1, 2) at its
@@ -319,9 +321,9 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
   }
   for (int i = tid; i < 2 * N * 4; i += TM_THREADS) s_mask[i] = 0u;
   if (tid == 0) *s_tiles = 0;
-  if (BOUND && bmask) __syncthreads();
+  if (MASKED) __syncthreads();
   griddep_wait();  // the rotated queries (and allow bitmaps, TQ+ terms) are written
-  if (BOUND && bmask) {
+  if (MASKED) {
     const int per = TM_M / fblock;  // 2 or 4 filter blocks a tile, in one mask word
     for (int i = tid; i < all_tiles; i += TM_THREADS) {
       const int t = (int)blockIdx.x + i * (int)gridDim.x, b = t * per;
@@ -404,7 +406,7 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (BOUND && bmask) my_tiles = *s_tiles;
+  if (MASKED) my_tiles = *s_tiles;
   const int total_ld = my_tiles * raws, total_it = my_tiles * blks;
 
   if (warp == TM_PROD) {
@@ -727,9 +729,9 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
 // (k_scan_stream's operations in its order) and the k best of those are the
 // result, unless a full list's last U reaches the k-th best score: a vector
 // that list dropped might belong to the result, so the gate opens.
-constexpr int RS_NT = 512;
+constexpr int RS_NT = 1024;
 constexpr int RS_CAP = 1024;  // candidates one block scores
-constexpr int RS_PER = 10;    // list entries per thread: 152 lists of 32
+constexpr int RS_PER = 5;     // list entries per thread: 152 lists of 32
 
 // (The kernel is one short block per query, so its time is latency: few
 // dependent round trips, and rolled loops, since the instructions come from L2
@@ -933,7 +935,8 @@ cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* ce
     return launch_maybe_pdl(pdl, kernel, grid, block, smem, s, map, qrot, centroids, scale, del, dense, allow_bits,
                             words, bmask, mask_words, fblock, bias, (int)n, (int)nq, d, k, C, cst, cand_s, cand_i, err, force, gth, lows);
   };
-  e = bound ? go(k_scan_tm<16, true>) : N == 16 ? go(k_scan_tm<16, false>) : go(k_scan_tm<32, false>);
+  e = bound ? (bmask ? go(k_scan_tm<16, true, true>) : go(k_scan_tm<16, true, false>))
+            : N == 16 ? go(k_scan_tm<16, false, false>) : go(k_scan_tm<32, false, false>);
   if (e != cudaSuccess) return e;
   if (ev1 && (e = cudaEventRecord(ev1, s)) != cudaSuccess) return e;
   return cudaSuccess;
