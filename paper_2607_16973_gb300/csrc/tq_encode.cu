@@ -15,6 +15,7 @@
 
 #include "tq_internal.h"
 #include "tq_kernels.h"
+#include "tq_topk.cuh"
 
 namespace tq {
 namespace {
@@ -481,7 +482,8 @@ __global__ void k_calib_finish(const double* __restrict__ psum, const double* __
 __global__ void __launch_bounds__(256)
 k_calib_query(float* __restrict__ qrot, int64_t nq, int d, const float* __restrict__ mu,
               const float* __restrict__ a, float* __restrict__ bias) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  griddep_launch_dependents();
+  griddep_wait();  // the rotated queries are written
   __shared__ float red[8];
   const int64_t q = blockIdx.x;
   float* qq = qrot + q * d;
@@ -631,8 +633,7 @@ cudaError_t launch_calibrate(const float* X, int64_t n, int d, const float* R, f
 cudaError_t launch_calib_query(float* qrot, int64_t nq, int d, const float* mu, const float* a, float* bias,
                                cudaStream_t s) {
   if (nq == 0) return cudaSuccess;
-  k_calib_query<<<(unsigned)nq, 256, 0, s>>>(qrot, nq, d, mu, a, bias);
-  return cudaGetLastError();
+  return launch_maybe_pdl(s != nullptr, k_calib_query, dim3((unsigned)nq), dim3(256), 0, s, qrot, nq, d, mu, a, bias);
 }
 
 }  // namespace tq

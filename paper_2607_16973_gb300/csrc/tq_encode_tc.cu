@@ -48,6 +48,7 @@
 #include "tq_internal.h"
 #include "tq_kernels.h"
 #include "tq_tc.cuh"
+#include "tq_topk.cuh"
 
 namespace tq {
 namespace {
@@ -477,6 +478,7 @@ k_rotate_tc(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CU
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 16) + 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x, p = blockIdx.y, sp = blockIdx.z;
+  griddep_launch_dependents();  // the next kernel's launch overlaps this one; it waits before reading
   const int KB = d / EK;
   const int kb0 = (int)((long long)sp * KB / S), nk = (int)((long long)(sp + 1) * KB / S) - kb0;
   if (tid == 0) {
@@ -599,7 +601,8 @@ k_rotate_tc(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CU
 __global__ void __launch_bounds__(256)
 k_rotate_reduce(const float4* __restrict__ part, int S, int64_t n4, float4* __restrict__ out, int* counters,
                 int64_t n_counters) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  griddep_launch_dependents();
+  griddep_wait();  // the partial products are written
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (counters)
@@ -744,9 +747,9 @@ cudaError_t launch_rotate_tc(const float* Q, int64_t nq, int d, const float* R, 
                                       : cudaSuccess;
   const int64_t n4 = nq * d / 4;
   const int blocks = (int)std::min<int64_t>((n4 + 255) / 256, (int64_t)device_sm_count() * 8);
-  k_rotate_reduce<<<std::max(blocks, 1), 256, 0, s>>>(reinterpret_cast<const float4*>(part), S, n4,
-                                                       reinterpret_cast<float4*>(out), counters, n_counters);
-  return cudaGetLastError();
+  return launch_maybe_pdl(s != nullptr, k_rotate_reduce, dim3(std::max(blocks, 1)), dim3(256), 0, s,
+                          reinterpret_cast<const float4*>(part), S, n4, reinterpret_cast<float4*>(out), counters,
+                          n_counters);
 }
 
 }  // namespace tq

@@ -14,7 +14,7 @@
 //   warps 8-15  epilogue: read the 128 x 256 fp32 accumulators from TMEM (one
 //               query per thread; warps 8-11 the first query tile, 12-15 the
 //               second), apply the per-vector scale and keep each query's
-//               top-k in a thread-private sorted list (rows marked in the
+//               top-k in a thread-private list (rows marked in the
 //               optional tombstone bitmap never enter it);
 //   warp 16     code producer: TMA of the code tiles; allocates TMEM;
 //   warp 17     MMA issuer: one thread issues tcgen05.mma (M=128, N=256,
@@ -38,6 +38,7 @@
 #include "tq_kernels.h"
 #include "tq_wait.cuh"
 #include "tq_tc.cuh"
+#include "tq_topk.cuh"
 
 namespace tq {
 namespace {
@@ -110,7 +111,7 @@ __device__ __forceinline__ float key_score(uint64_t key) { return ordered((uint3
 __device__ __forceinline__ int key_id(uint64_t key) { return (int)~(uint32_t)key; }
 
 struct MmaSmem {
-  uint32_t a, b, raw, tab, scale, dense, bars, total;
+  uint32_t a, b, raw, tab, scale, dense, bars, lists, total;
 };
 
 template <int BITS>
@@ -152,6 +153,7 @@ __host__ __device__ inline MmaSmem mma_smem_layout(int cst, int ast, int rr, int
   off = (off + 15) & ~15u;
   L.bars = off;
   off += 48 * 8;
+  L.lists = off;  // the lists follow where they fit (list_bytes), else they are in global memory
   L.total = off + 1024;  // slack to align the base to 1024 bytes
   // at most one CTA per SM: each allocates all 512 TMEM columns
   if (L.total < 116u * 1024u) L.total = 116u * 1024u;
@@ -253,7 +255,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
            const uint32_t* __restrict__ allow_bits, int words, const float* __restrict__ bias, int n, int nq,
            int d, int k, int cst, int ast, int rr, int sub, int ng, int gact, float* __restrict__ cand_s,
            int* __restrict__ cand_i, int* __restrict__ err, uint32_t* __restrict__ gth,
-           uint32_t* heads, uint64_t* __restrict__ lists) {
+           uint32_t* heads, uint64_t* lists) {
   constexpr int RAWB = raw_bytes_per_row<BITS>();
   // A code tile carries `sub` consecutive K-blocks of 256 rows: rows of
   // sub*RAWB bytes (128 B, one full line, when d allows), stored with the
@@ -348,6 +350,8 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int total_it = my_tiles * kblocks;
+  griddep_launch_dependents();
+  griddep_wait();  // the packed queries, allow bitmaps and zeroed thresholds are written
 
   if (warp == CODE_WARP) {
     // ------------------------------------------------- code tiles (TMA, HBM)
@@ -517,14 +521,15 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
     // a filtered search: this query's allow bitmap over the dense tenant index
     const uint32_t* ab = allow_bits && q < nq ? allow_bits + (size_t)q * words : nullptr;
     const float bq = bias && q < nq ? bias[q] : 0.f;  // a TQ+ index's per-query term (else 0)
-    // This query's k best so far: keys in no order, and the worst of them.  They
-    // live in global memory (L1 and L2), not in shared memory, whose room they
-    // took from the decoded tiles' stages (k = 10: two decoder groups instead of
-    // three), and are not kept sorted: a new entry replaces the worst and the
-    // list is read once, k independent loads, for the next worst.  Shifting a
-    // sorted list entry by entry cost about 60 cycles each: 300 of the 430 us of
-    // 50 queries, k = 20, over 300,001 x 1024.
-    uint64_t* lst = lists + (((size_t)blockIdx.y * gridDim.x + blockIdx.x) * QT + jsel) * k * MMA_M + row;
+    // This query's k best so far: keys in no order, and the worst of them, in
+    // shared memory where the plan leaves room, else in global memory (L1 and
+    // L2; `lists`): in shared memory at any price they took a decoder group's
+    // stage (k = 10). A new entry replaces the worst and the list is read once, k
+    // independent loads, for the next worst.  Shifting a sorted list entry by
+    // entry cost about 60 cycles each: 300 of the 430 us of 50 queries, k = 20,
+    // over 300,001 x 1024.
+    uint64_t* lst = lists ? lists + (((size_t)blockIdx.y * gridDim.x + blockIdx.x) * QT + jsel) * k * MMA_M + row
+                          : reinterpret_cast<uint64_t*>(base + L.lists) + jsel * k * MMA_M + row;
     uint64_t worst = 0;  // 0: not full yet
     int cnt = 0, wslot = 0;
     float th_s = -INFINITY;
@@ -533,10 +538,11 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
     float th_g = -INFINITY, th = -INFINITY;  // th = max(th_s, th_g)
     float ps0 = 0.f, ps1 = 0.f, ps2 = 0.f, ps3 = 0.f;  // parked candidates of the current tile
     int pi0 = 0, pi1 = 0, pi2 = 0, pi3 = 0, npark = 0;
-    // tiles before which the CTAs' best scores are read, and after whose
-    // predecessors they are published
+    // tiles before which the CTAs' heads are read, and after whose predecessors
+    // they are published: a CTA's best score or, for k > 32, its rank-th best
+    const int rank = k <= 32 ? 1 : (k + 15) / 16, reach = (k + rank - 1) / rank;
     auto heads_turn = [&](int tile_i) {
-      return (tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= 8 && k <= 32 && (int)gridDim.x >= k;
+      return (tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= 8 && (int)gridDim.x >= reach;
     };
     auto insert = [&](float sc, int v) {
       const uint64_t key = rank_key(sc, v);
@@ -546,7 +552,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       if (cnt < k) ++cnt;
       if (cnt < k) return;
       worst = ~0ull;
-#pragma unroll 4
+#pragma unroll 8
       for (int i = 0; i < k; ++i) {
         const uint64_t o = i == slot ? key : lst[i * MMA_M];  // (not waiting for the store)
         wslot = o < worst ? i : wslot;
@@ -567,8 +573,9 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       }
       const uint32_t shared_th = mine && q < nq ? __ldcg(gth + q) : 0u;
       if (heads_turn(tile_i) && mine && q < nq) {
-        // Every CTA has published its best score for the query.  The k-th best of
-        // the maxima of 32 groups of CTAs is reached by k vectors; with all
+        // Every CTA has published its best (rank-th best) score for the query.
+        // The k-th (k / rank-th) best of the maxima of 32 groups of CTAs is
+        // reached by k vectors; with all
         // CTAs' rows behind it, few vectors of a tile reach it (a CTA's own
         // list is beaten by k / i vectors of its tile i).  It costs about 5 us, so
         // not for a small k: 300,001 x 1024, 50 queries: k = 20 281 -> 238 us, k = 5
@@ -588,7 +595,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
           int have = 0;
 #pragma unroll
           for (int i = 0; i < 32; ++i) have += g[i] >= up ? 1 : 0;
-          b = have >= k ? up : b;
+          b = have >= reach ? up : b;
         }
         if (b) th_g = fmaxf(th_g, ordered(b));
       }
@@ -607,42 +614,78 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       if (mine) {
         const uint32_t tb = tmem + ((uint32_t)(32 * e) << 16) + (uint32_t)((set * QT + jsel) * NT);
         if (shared_th) th_g = fmaxf(th_g, ordered(shared_th));
-        if (tile_i == 0 && !allow_bits && n - v0 >= NT) {
+        if (tile_i == 0 && !allow_bits) {
           // The first tile's vectors all pass an empty list's threshold, and
           // taking up to 256 of them into the list one by one took longer than
-          // many tiles' MMAs (k = 20: about 100 us).  So the list first takes
-          // the maxima of groups of 8 columns (4 for k > 32): k of those are
-          // distinct vectors, so their k-th best is a first threshold, which
-          // about k vectors of the tile reach.
-          const bool fine = k > 32;
+          // many tiles' MMAs (k = 20: about 100 us).  So a first threshold comes
+          // from the tile itself.  For k <= 16: the list takes the maxima of
+          // groups of 8 columns, and the k-th best of them, k distinct vectors'
+          // scores, is one.  For larger k: the tile's scores are counted
+          // against a threshold bisected between their extremes.
+          auto each = [&](auto&& fn) {  // fn(c0, 16 scores) by chunk, -infinity for rows deleted or past n
 #pragma unroll 1
-          for (int c0 = 0; c0 < NT; c0 += 16) {
-            uint32_t r[16];
-            tmem_ld16_issue(tb + (uint32_t)c0, r);
-            tmem_wait16(r);
-            if (q >= nq) continue;
-            const uint32_t dead = del ? __ldg(del + ((v0 + c0) >> 5)) >> (c0 & 16) : 0u;
-            float m4[4];
+            for (int c0 = 0; c0 < NT; c0 += 16) {
+              uint32_t r[16];
+              tmem_ld16_issue(tb + (uint32_t)c0, r);
+              tmem_wait16(r);
+              const int rows = n - (v0 + c0);
+              uint32_t dead = rows >= 16 ? 0u : rows > 0 ? 0xFFFFu << rows : 0xFFFFu;
+              if (del && rows > 0) dead |= __ldg(del + ((v0 + c0) >> 5)) >> (c0 & 16);
+              float x[16];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float4 s4 = *reinterpret_cast<const float4*>(sScale + c0 + 4 * j);
-              const float x[4] = {(__uint_as_float(r[4 * j]) + bq) * s4.x, (__uint_as_float(r[4 * j + 1]) + bq) * s4.y,
-                                  (__uint_as_float(r[4 * j + 2]) + bq) * s4.z,
-                                  (__uint_as_float(r[4 * j + 3]) + bq) * s4.w};
-              m4[j] = -INFINITY;
+              for (int j = 0; j < 16; j += 4) {
+                const float4 s4 = *reinterpret_cast<const float4*>(sScale + c0 + j);
+                x[j] = (__uint_as_float(r[j]) + bq) * s4.x;
+                x[j + 1] = (__uint_as_float(r[j + 1]) + bq) * s4.y;
+                x[j + 2] = (__uint_as_float(r[j + 2]) + bq) * s4.z;
+                x[j + 3] = (__uint_as_float(r[j + 3]) + bq) * s4.w;
+              }
 #pragma unroll
-              for (int i = 0; i < 4; ++i) m4[j] = fmaxf(m4[j], (dead >> (4 * j + i)) & 1u ? -INFINITY : x[i]);
+              for (int j = 0; j < 16; ++j) x[j] = (dead >> j) & 1u ? -INFINITY : x[j];
+              fn(c0, x);
             }
+          };
+          if (k <= 16) {
+            each([&](int c0, const float (&x)[16]) {
+              if (q >= nq) return;
 #pragma unroll 1
-            for (int j = fine ? 0 : 1; j < 4; j += fine ? 1 : 2) {
-              const float pair = fmaxf(j == 1 ? m4[0] : m4[2], j == 1 ? m4[1] : m4[3]);
-              insert(fine ? (j == 0 ? m4[0] : j == 1 ? m4[1] : j == 2 ? m4[2] : m4[3]) : pair, c0 + 4 * j);
+              for (int j = 0; j < 2; ++j) {
+                float best = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) best = (i >> 3) == j ? fmaxf(best, x[i]) : best;
+                insert(best, c0 + 8 * j);
+              }
+            });
+            th_g = fmaxf(th_g, th_s);
+            worst = 0;
+            cnt = 0;
+            th_s = -INFINITY;
+          } else {
+            float lo = INFINITY, hi = -INFINITY;
+            int live = 0;
+            each([&](int, const float (&x)[16]) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                live += x[i] > -INFINITY ? 1 : 0;
+                lo = x[i] > -INFINITY ? fminf(lo, x[i]) : lo;
+                hi = fmaxf(hi, x[i]);
+              }
+            });
+            const bool enough = live >= k;  // k of them reach lo, then
+#pragma unroll 1
+            for (int pass = 0; pass < 9; ++pass) {
+              const float mid = 0.5f * lo + 0.5f * hi;
+              int have = 0;
+              each([&](int, const float (&x)[16]) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) have += x[i] >= mid ? 1 : 0;
+              });
+              lo = have >= k ? mid : lo;
+              hi = have >= k ? hi : mid;
+              if (__all_sync(0xffffffffu, !enough || (have >= k && have <= k + 2))) break;
             }
+            if (enough) th_g = fmaxf(th_g, lo);
           }
-          th_g = fmaxf(th_g, th_s);
-          worst = 0;
-          cnt = 0;
-          th_s = -INFINITY;
           __syncwarp();
         }
         th = fmaxf(th_s, th_g);
@@ -730,25 +773,39 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
         if (b > shared_th) atomicMax(gth + q, b);
       }
       if (heads_turn(tile_i + 1) && mine && q < nq) {
-        uint64_t best = 0;
-        for (int i = 0; i < cnt; ++i) best = max(best, lst[i * MMA_M]);
-        heads[(size_t)blockIdx.x * nq + q] = (uint32_t)(best >> 32);
+        uint64_t last = ~0ull;
+        for (int r = 0; r < rank; ++r) {
+          uint64_t best = 0;
+#pragma unroll 4
+          for (int i = 0; i < cnt; ++i) {
+            const uint64_t o = lst[i * MMA_M];
+            best = o < last && o > best ? o : best;
+          }
+          last = best;
+        }
+        heads[(size_t)blockIdx.x * nq + q] = (uint32_t)(last >> 32);
       }
       asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
     }
     if (mine && q < nq) {
-      uint64_t last = ~0ull;  // written best first: each round takes the best key below the last one's
-      for (int r = 0; r < k; ++r) {
-        uint64_t best = 0;
+      // the list, its best entry first and its worst (or an empty one) last, as
+      // the merge takes its bounds; the others in any order
+      uint64_t best = 0;
+      int bi = 0;
+#pragma unroll 8
+      for (int i = 0; i < cnt; ++i) {
+        const uint64_t o = lst[i * MMA_M];
+        bi = o > best ? i : bi;
+        best = o > best ? o : best;
+      }
+      const size_t o0 = ((size_t)q * gridDim.x + blockIdx.x) * k;
+      int p = 1;
 #pragma unroll 4
-        for (int i = 0; i < cnt; ++i) {
-          const uint64_t o = lst[i * MMA_M];
-          best = o < last && o > best ? o : best;
-        }
-        const size_t o = ((size_t)q * gridDim.x + blockIdx.x) * k + r;
-        cand_s[o] = best ? key_score(best) : -INFINITY;
-        cand_i[o] = best ? key_id(best) : INT_MAX;
-        last = best;
+      for (int i = 0; i < k; ++i) {
+        const uint64_t key = i < cnt ? lst[i * MMA_M] : 0;
+        const int at = i < cnt ? (i == bi ? 0 : cnt == k && i == wslot ? k - 1 : p++) : i;
+        cand_s[o0 + at] = key ? key_score(key) : -INFINITY;
+        cand_i[o0 + at] = key ? key_id(key) : INT_MAX;
       }
     }
   }
@@ -761,6 +818,8 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
 // Rotated queries (float32 [nq, d]) -> fp16 A blocks [qtile][kblock][128 x 64],
 // K-major with the 128-byte swizzle, rows past nq zero.
 __global__ void k_pack_queries(const float* __restrict__ qrot, int nq, int d, __half* __restrict__ out) {
+  griddep_launch_dependents();
+  griddep_wait();  // the rotated queries are written
   const int kblocks = d / KB;
   const int qt = blockIdx.y, kb = blockIdx.x;
   unsigned char* dst = reinterpret_cast<unsigned char*>(out) + ((size_t)qt * kblocks + kb) * A_BYTES;
@@ -784,16 +843,21 @@ template <int BITS, int QT>
 cudaError_t launch_typed(const MmaPlan& P, const CUtensorMap& map, const __half* qpack, const float* centroids,
                          const float* scale, const uint32_t* del, const uint32_t* dense, const uint32_t* allow,
                          int words, const float* bias, int n, int nq, int d, int k, int sub, int grid_x, float* cs,
-                         int* ci, int* err, uint32_t* gth, uint32_t* heads, uint64_t* lists, cudaStream_t s) {
+                         int* ci, int* err, uint32_t* gth, uint32_t* heads, uint64_t* lists, bool pdl, cudaStream_t s) {
+  uint32_t smem = P.smem;
+  const uint32_t room = (uint32_t)QT * k * MMA_M * sizeof(uint64_t);
+  if (smem + room <= kMaxDynSmem) {
+    smem += room;
+    lists = nullptr;
+  }
   const int gact = active_groups(P.ng, sub, P.cst);
-  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_scan_mma<BITS, QT>), (int)P.smem);
+  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_scan_mma<BITS, QT>), (int)smem);
   if (e != cudaSuccess) return e;
   const int nqt = (nq + MMA_M - 1) / MMA_M;
   const dim3 grid((unsigned)grid_x, (unsigned)((nqt + QT - 1) / QT));
-  k_scan_mma<BITS, QT><<<grid, NTHREADS, P.smem, s>>>(map, qpack, centroids, scale, del, dense, allow, words, bias,
-                                                         n, nq, d, k, P.cst, P.ast, P.rr, sub, P.ng, gact, cs, ci,
-                                                         err, gth, heads, lists);
-  return cudaGetLastError();
+  return launch_maybe_pdl(pdl, k_scan_mma<BITS, QT>, grid, dim3(NTHREADS), (size_t)smem, s, map, qpack, centroids,
+                          scale, del, dense, allow, words, bias, n, nq, d, k, P.cst, P.ast, P.rr, sub, P.ng, gact, cs,
+                          ci, err, gth, heads, lists);
 }
 
 MmaPlan plan_for(int bits, int64_t nq) {
@@ -858,17 +922,18 @@ cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* c
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   const dim3 pgrid((unsigned)(d / KB), (unsigned)((nq + MMA_M - 1) / MMA_M));
-  k_pack_queries<<<pgrid, 256, 0, s>>>(qrot, (int)nq, d, static_cast<__half*>(qpack));
-  cudaError_t e = cudaGetLastError();
+  const bool pdl = s != nullptr && ev0 == nullptr;
+  cudaError_t e = launch_maybe_pdl(s != nullptr, k_pack_queries, pgrid, dim3(256), 0, s, qrot, (int)nq, d,
+                                   static_cast<__half*>(qpack));
   if (e != cudaSuccess) return e;
   if (ev0 && (e = cudaEventRecord(ev0, s)) != cudaSuccess) return e;
   const __half* qp = static_cast<const __half*>(qpack);
 #define TQ_MMA_CASE(B)                                                                                \
   case B:                                                                                             \
     e = P.qt == 2 ? launch_typed<B, 2>(P, map, qp, centroids, scale, del, dense, allow_bits, words, bias, \
-                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, gth, heads, lists, s)        \
+                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, gth, heads, lists, pdl, s)        \
                   : launch_typed<B, 1>(P, map, qp, centroids, scale, del, dense, allow_bits, words, bias, \
-                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, gth, heads, lists, s);       \
+                                       (int)n, (int)nq, d, k, sub, grid_x, cand_s, cand_i, err, gth, heads, lists, pdl, s);       \
     break;
   switch (bits) {
     TQ_MMA_CASE(2)

@@ -823,6 +823,7 @@ k_merge_lists(const float* __restrict__ cand_s, const int* __restrict__ cand_i, 
   int* wi = reinterpret_cast<int*>(ws + (blockDim.x >> 5) * k);
   unsigned char* scratch = reinterpret_cast<unsigned char*>(wi + (blockDim.x >> 5) * k);
   const int64_t q = blockIdx.x;
+  griddep_wait();  // the lists are written
   merge_lists_block(cand_s + q * nlists * k, cand_i + q * nlists * k, nlists, k, ext, out_ids + q * k,
                     out_scores + q * k, ws, wi, scratch, scratch_bytes);
 }
@@ -1132,9 +1133,8 @@ cudaError_t launch_merge(const float* cand_s, const int32_t* cand_i, int64_t nq,
   // (dynamic plus the kernel's few static bytes stay under the default 48 KB)
   const size_t scratch = std::min<size_t>(want, 40 * 1024 - (size_t)warps * k * 8);
   const size_t smem = (size_t)warps * k * (sizeof(float) + sizeof(int32_t)) + scratch;
-  k_merge_lists<<<(unsigned)nq, 32 * warps, smem, s>>>(cand_s, cand_i, nlists, k, ext, out_ids, out_scores,
-                                                       scratch);
-  return cudaGetLastError();
+  return launch_maybe_pdl(s != nullptr, k_merge_lists, dim3((unsigned)nq), dim3(32 * warps), smem, s, cand_s, cand_i,
+                          nlists, k, ext, out_ids, out_scores, scratch);
 }
 
 cudaError_t launch_merge_global(const float* cand_s, const int64_t* cand_i, int64_t S, int64_t nq, int64_t m,

@@ -198,8 +198,9 @@ __device__ bool merge_lists_small(const float* cs, const int* ci, int nlists, in
   return true;
 }
 
-// Merge of per-CTA candidate lists that are each sorted best first and hold
-// exactly k entries (padding (-inf, INT_MAX) at the end).  The k-th entry T of
+// Merge of per-CTA candidate lists that hold exactly k entries each, their
+// best first and their worst last (padding (-inf, INT_MAX) at the end); the
+// lookup scans' are sorted.  The k-th entry T of
 // any one list is beaten or matched by that list's k entries, so the global
 // k-th best is at least as good as the best such T and worse candidates are
 // skipped at once.  Each warp keeps a sorted top-k of its share of the rest

@@ -1,5 +1,5 @@
 """The batched tensor-core scan's lists and thresholds (k_scan_mma): a first
-threshold from the first tile's column groups (of 8 columns, of 4 for k > 32),
+threshold from the first tile (group maxima, or a bisection for k > 16),
 thresholds and list heads shared between the CTAs of a query (several tiles
 per CTA), with deleted rows, ties and fewer live rows than k."""
 import numpy as np
@@ -20,11 +20,11 @@ def tdev(cuda_lib):
 
 
 @pytest.mark.parametrize("n,nq,k,bits,dead", [
-    (256, 40, 64, 4, 0.0),         # one whole tile, groups of 4 columns
-    (255, 33, 20, 2, 0.0),         # a short tile: no first threshold
+    (256, 40, 64, 4, 0.0),         # one whole tile
+    (255, 33, 20, 2, 0.0),         # a short tile
     (90_001, 40, 20, 4, 0.3),      # three tiles per CTA: heads read at the second; deleted rows
     (90_001, 130, 8, 2, 0.0),      # two query tiles, the smallest k that reads heads
-    (60_000, 300, 33, 4, 0.999),   # groups of 4, fewer live rows per CTA than k
+    (60_000, 300, 33, 4, 0.999),   # fewer live rows per CTA than k; heads of rank 3
 ])
 def test_mma_lists(cuda_lib, tdev, n, nq, k, bits, dead):
     torch, T = tdev
