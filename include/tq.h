@@ -197,7 +197,10 @@ tq_status tq_encode_ex(const float* X, int64_t n, int d, const float* R,
  *                rate), again in three products of operands split in two, each
  *                row of X and R scaled by a power of two first.  fp16 keeps the
  *                same 10 mantissa bits as TF32, so the error is no larger; the
- *                calls may land boundary coordinates in different cells.  The
+ *                calls may land boundary coordinates in different cells.
+ *                (From d = 1024 on, 8-bit codes from 768; below, where such
+ *                a coordinate weighs more in its row's scalar, it runs as
+ *                tq_encode_planned and reads no workspace.)  The
  *                workspace is free again when the call's work has finished.
  *                n up to 2^31 - 1024.
  */

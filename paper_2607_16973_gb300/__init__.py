@@ -118,7 +118,8 @@ def encode(X, R, centroids, boundaries, bits: int, scale_mode: str = "norm",
             _dev_ptr(codes, "codes", torch.uint8), _dev_ptr(scale, "scale", f32))
     handle = _stream_handle(stream)
     if plan is not None:
-        need = encode_workspace(n, d)
+        # below these d the fp16 encoder does not run and reads no workspace
+        need = encode_workspace(n, d) if d >= (768 if bits == 8 else 1024) else None
         if workspace is None and need is not None:
             try:
                 with _on_stream(stream):

@@ -210,8 +210,12 @@ extern "C" tq_status tq_encode_planned_ws(const float* X, int64_t n, int d, cons
   if (!workspace || !tq::aligned16(workspace))
     return fail(TQ_EINVAL, "tq_encode_planned_ws: the workspace must be 16-byte aligned device memory");
   if (ws_bytes < need) return fail(TQ_EINVAL, "tq_encode_planned_ws: workspace of %zu bytes, %zu needed", ws_bytes, need);
-  const cudaError_t e = tq::launch_encode_h(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a,
-                                            codes, scale, workspace, (cudaStream_t)stream);
+  const cudaError_t e =
+      tq::encode_h_applies(d, bits)
+          ? tq::launch_encode_h(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a, codes, scale,
+                                workspace, (cudaStream_t)stream)
+          : tq::launch_encode_tc(X, n, d, plan, centroids, boundaries, bits, scale_mode, cal_mu, cal_a, codes, scale,
+                                 (cudaStream_t)stream);
   if (e != cudaSuccess) return tq::cuda_fail("tq_encode_planned_ws", e);
   return tq::ok();
 }

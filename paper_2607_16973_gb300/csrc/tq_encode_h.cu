@@ -604,13 +604,23 @@ int encode_h_chunk(int64_t n, int d) {
 
 }  // namespace
 
-size_t encode_h_workspace(int64_t n, int d) { return h_ws(n, d).total; }
+// Where the fp16 encoder runs.  The two encoders decide about 2 in 100,000
+// coordinates, those next to a boundary, differently, and one such coordinate
+// moves its row's scalar by (c1^2 - c0^2) / 2, at the outermost boundary up to
+// 1.04 / d of its value for 2-bit, 1.4 / d for 3-bit, 1.6 / d for 4-bit codes,
+// times its calibration squared.  Over 999,000 rows the largest change of a
+// scalar measured was 4.1e-3 at d = 768, 3.0e-3 at 1024, 2.1e-3 at 1536.  The
+// outer boundaries of 8-bit codes are rarely reached (2.2e-3 at d = 768).  Below
+// these d the codes stay those of the TF32 encoder.
+bool encode_h_applies(int d, int bits) { return encode_tc_supported(d) && d >= (bits == 8 ? 768 : 1024); }
+
+size_t encode_h_workspace(int64_t n, int d) { return encode_h_applies(d, 8) ? h_ws(n, d).total : 256; }
 
 cudaError_t launch_encode_h(const float* X, int64_t n, int d, const void* plan, const float* centroids,
                             const float* boundaries, int bits, int scale_mode, const float* cal_mu,
                             const float* cal_a, uint8_t* codes, float* scale, void* ws, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  if (!encode_tc_supported(d)) return cudaErrorInvalidValue;
+  if (!encode_h_applies(d, bits)) return cudaErrorInvalidValue;
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
   if (!enc) return cudaErrorNotSupported;
   const HWs w = h_ws(n, d);

@@ -38,6 +38,7 @@ cudaError_t launch_encode_tc(const float* X, int64_t n, int d, const void* plan,
 
 // The same in fp16 (three products of operands split in two, rows scaled by
 // powers of two), with a workspace of encode_h_workspace(n, d) bytes.
+bool encode_h_applies(int d, int bits);
 size_t encode_h_workspace(int64_t n, int d);
 cudaError_t launch_encode_h(const float* X, int64_t n, int d, const void* plan, const float* centroids,
                             const float* boundaries, int bits, int scale_mode, const float* cal_mu,

@@ -34,11 +34,11 @@ def _tf32(tq, torch, X, plan, c, t, bits, mode):
 
 
 @pytest.mark.parametrize("n,d,bits,mode", [
-    (1, 128, 4, "norm"),           # one row, one chunk
-    (129, 160, 3, "unbiased"),     # a row past a panel; a partial chunk
+    (1, 1024, 4, "norm"),           # one row, the smallest d
+    (129, 1056, 3, "unbiased"),     # a row past a panel; a partial chunk
     (1_000, 1536, 4, "norm"),      # fewer items than SMs
     (2_500, 1536, 8, "none"),      # 20 panels
-    (19_700, 384, 2, "norm"),      # 154 panels: one item over the SMs, panels split between CTAs
+    (19_700, 1024, 2, "norm"),     # 154 panels split between CTAs, a partial chunk
 ])
 def test_encode_h_parity(cuda_lib, tdev, n, d, bits, mode):
     torch, dev, T = tdev
@@ -68,7 +68,7 @@ def test_encode_h_values_out_of_range(cuda_lib, tdev):
     TF32 encoder; a matrix R of another scale is brought into fp16's range."""
     torch, dev, T = tdev
     tq = cuda_lib
-    n, d, bits = 300, 256, 4
+    n, d, bits = 300, 1024, 4
     X = synth.gaussian_rows(n, d, seed=3)
     X[10, 5] = np.inf
     X[11, 6] = np.nan
@@ -94,7 +94,7 @@ def test_encode_h_workspace(cuda_lib, tdev):
     """A kept workspace is reused, one that is too small is refused."""
     torch, dev, T = tdev
     tq = cuda_lib
-    n, d, bits = 700, 512, 4
+    n, d, bits = 700, 1024, 4
     R = O.rotation(d, 7).astype(np.float32)
     c32, t32 = _cb(d, bits)
     plan = tq.encode_plan(T(R))
@@ -107,3 +107,15 @@ def test_encode_h_workspace(cuda_lib, tdev):
     with pytest.raises(tq.TQError):
         tq.encode(X[0], None, T(c32), T(t32), bits, plan=plan, workspace=ws[:-1])
     assert tq.encode_workspace(n, 96) is None
+
+
+@pytest.mark.parametrize("d,bits", [(384, 3), (992, 4), (736, 8)])
+def test_below_its_range_the_tf32_encoder_runs(cuda_lib, tdev, d, bits):
+    torch, dev, T = tdev
+    tq = cuda_lib
+    X, R = T(synth.gaussian_rows(500, d, seed=d)), O.rotation(d, 7).astype(np.float32)
+    c32, t32 = (T(a) for a in tq.codebook(d, bits)[:2])
+    plan = tq.encode_plan(T(R))
+    codes, scale = tq.encode(X, None, c32, t32, bits, plan=plan)
+    codes_t, scale_t = _tf32(tq, torch, X, plan, c32, t32, bits, "norm")
+    assert np.array_equal(codes.cpu().numpy(), codes_t) and np.array_equal(scale.cpu().numpy(), scale_t)
