@@ -100,11 +100,23 @@ def source_hash(*files):
     return h.hexdigest()[:16]
 
 
-def lookup_kernel(bits: int, n: int, d: int, k: int) -> str:
-    """The lookup scan tq_search's AUTO path runs below the tensor-core batch
-    size: the bulk-copy ring for 3-bit codes, else the register-fed byte-pair
-    (4-bit) or per-code scan."""
+def small_batch_kernel(bits: int, n: int, d: int, k: int, nq: int = 1, path: str = "auto") -> str:
+    """The scan tq_search runs for an unfiltered batch below 16 queries: the
+    small-batch tensor-core scan (exact: its candidates are rescored in float32)
+    for 4-bit codes and enough work, else a lookup scan: the bulk-copy ring for
+    3-bit codes, the register-fed byte-pair (4-bit) or per-code scan otherwise."""
+    if path == "lut_fold":
+        return "k_scan_fold"
+    if path == "auto" and bits == 4 and d % 256 == 0 and d <= 2048 and k <= 32 and n >= 2048 and \
+            n * d * nq >= (1 << 24 if k <= 16 else 1 << 27):
+        return "k_scan_tm"
     return "k_scan_ring" if bits == 3 else "k_scan_stream"
+
+
+def fp16_kernel(bits: int, d: int, k: int, nq: int, path: str = "auto") -> str:
+    """The tensor-core scan of a batch of 16 or more queries."""
+    small = path == "auto" and nq <= 32 and bits == 4 and d % 256 == 0 and d <= 2048 and k <= 32
+    return "k_scan_tm" if small else "k_scan_mma"
 
 
 def recorded_traffic(kernel_file, profile_md: str, scale_to: int):
@@ -477,15 +489,18 @@ def run_ours(args, cfg, rank, world):
                     "frac": achieved / peak, "frac_of": pk["source"] + " burst bf16 (= fp16 dense rate)",
                     "frac_of_sustained": achieved / pk["bf16_tflops_sustained"],
                     "traffic": recorded_traffic("paper_2607_16973_gb300/csrc/tq_mma.cu", "k_scan_mma_250k_batch1024.md",
-                                                scale_to=n),
-                    "kernel": "k_scan_mma", "alg_flops_per_launch": flops, "kernel_ms": scan_ms,
+                                                scale_to=n) if B >= 1024 else None,
+                    "kernel": fp16_kernel(bits, d, k, B, args.search_path), "alg_flops_per_launch": flops, "kernel_ms": scan_ms,
                     "hbm_gbs_of_corpus": alg_bytes / (scan_ms / 1e3) / 1e9}
         else:
             # lookup scan (with its last CTA's merge): the corpus, codes + scales,
             # read once per launch
             achieved = alg_bytes / (scan_ms / 1e3) / 1e9
-            kern = "k_scan_fold" if args.search_path == "lut_fold" else lookup_kernel(bits, n, d, k)
-            if kern == "k_scan_fold":
+            kern = small_batch_kernel(bits, n, d, k, B, args.search_path)
+            if kern == "k_scan_tm":
+                traffic = recorded_traffic("paper_2607_16973_gb300/csrc/tq_scan_tm.cu", "k_scan_tm_250k_batch1.md",
+                                           scale_to=n)
+            elif kern == "k_scan_fold":
                 traffic = recorded_traffic(("paper_2607_16973_gb300/csrc/tq_fold.cu",
                                             "paper_2607_16973_gb300/csrc/tq_topk.cuh"), "k_scan_fold_250k_batch1.md",
                                            scale_to=n)
@@ -532,8 +547,10 @@ def run_ours(args, cfg, rank, world):
         e2e_ms = a.elapsed_time(b)
         # our kernels per step: the rotation (with its reduce from 16 queries on:
         # the tensor-core rotation), then the lookup scan (merged in its last
-        # CTA) or query packing + tensor-core scan + merge; + the shard merge
-        launches = (2 if B >= 16 else 1) + (3 if mma else 1) + (1 if world > 1 else 0)
+        # CTA), or the bounding scan + rescoring + the lookup scan behind its
+        # gates, or (query packing +) tensor-core scan + merge; + the shard merge
+        scan_launches = {"k_scan_mma": 3, "k_scan_tm": 2 if mma else 3}.get(roof["kernel"], 1)
+        launches = (2 if B >= 16 else 1) + scan_launches + (1 if world > 1 else 0)
         results[B] = {
             "value": qps, "ms_per_step": ms / args.steps, "roofline": roof, "clocks": clk.summary(),
             "gpu_launches": launches * args.steps,
@@ -599,7 +616,7 @@ def run_ours(args, cfg, rank, world):
                              "roofline": v["roofline"], "e2e": v["e2e"], "gpu_launches": v["gpu_launches"]}
                     for b, v in results.items()},
         "encode": {"value": n / enc_ms * 1e3, "unit": "vectors/s", "ms": enc_ms,
-                   "path": "tensor core (TF32, three-product split)", "roofline": _roof_encode(n, d, enc_ms, pk),
+                   "path": "tensor core (fp16, three-product split)", "roofline": _roof_encode(n, d, enc_ms, pk),
                    "ffma": {"value": n / ffma_ms * 1e3, "unit": "vectors/s", "ms": ffma_ms,
                             "tflops": 2.0 * n * d * d / (ffma_ms / 1e3) / 1e12}},
     }
@@ -702,19 +719,16 @@ def _roof_tc(flops, ms, pk):
             "traffic": None, "kernel": "k_scan_mma", "alg_flops_per_launch": flops, "kernel_ms": ms}
 
 
-TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 / BF16 tensor rates of the GB300
-
-
 def _roof_encode(n, d, ms, pk):
-    """Roofline of the tensor-core encoder: three TF32 products per
-    multiply-add of the rotation (2 n d^2 flops each), against the TF32
-    peak taken as the measured burst bf16 peak times the nominal ratio."""
+    """Roofline of the tensor-core encoder: three fp16 products per
+    multiply-add of the rotation (2 n d^2 flops each), against the measured
+    burst bf16 peak (the same dense rate)."""
     flops = 3 * 2.0 * n * d * d
     tf = flops / (ms / 1e3) / 1e12
-    peak = pk["bf16_tflops"] * TF32_PER_BF16
+    peak = pk["bf16_tflops"]
     return {"bound": "tensor", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak,
-            "frac_of": pk["source"] + " burst bf16 x 1.1/2.25 (TF32 dense rate)", "traffic": None,
-            "kernel": "k_encode_tc", "alg_flops_per_launch": flops, "kernel_ms": ms,
+            "frac_of": pk["source"] + " burst bf16 (= fp16 dense rate)", "traffic": None,
+            "kernel": "k_encode_h", "alg_flops_per_launch": flops, "kernel_ms": ms,
             "rotation_tflops": 2.0 * n * d * d / (ms / 1e3) / 1e12}
 
 
@@ -778,8 +792,8 @@ def extras_100k(torch, tq, dev, stream, pk, flush, steps):
                     tq.set_search_path("auto")
                 ex = torch.topk(exact_sc, k, dim=1)[1]
             stream.synchronize()
-            roof = _roof_tc(2.0 * n * d * B, kms, pk) if B >= MMA_MIN_BATCH else _roof_hbm(alg, kms, pk,
-                                                                                        "k_scan_stream")
+            roof = _roof_tc(2.0 * n * d * B, kms, pk) if B >= MMA_MIN_BATCH else _roof_hbm(
+                alg, kms, pk, small_batch_kernel(bits, n, d, k, B))
             out[f"batch{B}_top{k}"] = {"value": B / ms * 1e3, "unit": "queries/s", "ms_per_step": ms,
                                        "roofline": roof, "recall": _recall(torch, got.cpu(), ex.cpu())}
             log(f"[bench] 100K batch {B} top-{k}: {B / ms * 1e3:.4g} q/s, scan {kms * 1e3:.1f} us")
@@ -1009,7 +1023,7 @@ def run_filtered(args, cfg):
             "config": {"workload": f"filtered: N={n} d={d} {bits}-bit top-{k}, Zipf tenants T in {cfg['tenants']}, "
                                    f"block {blk}, 10% of queries allow 5 tenants", "n": n, "d": d, "bits": bits,
                        "k": k, "block": blk},
-            "variants": variants, "gpu_launches": 4 * steps}
+            "variants": variants, "gpu_launches": 3 * steps}
     print(json.dumps(line), flush=True)
 
 

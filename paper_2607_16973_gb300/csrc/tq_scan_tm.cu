@@ -17,9 +17,10 @@
 // memory for the kernel's life (N x d fp16), so no query bytes are re-read per
 // tile.  (Decoding a quarter of the words with byte permutes instead of lookups,
 // to relieve that datapath, was slower, 185 us against 170: with 27 warps the
-// decoders are as close to the issue rate.)  Measured at 999,000 x 1536, whole searches: one query, top-5, 217 us
-// (lookup scan) -> 165; 32 queries 484 us (k_scan_mma) -> 216; eight queries
-// over 250,007 rows 425 us -> 115.
+// decoders are as close to the issue rate.)  Measured at 999,000 x 1536, whole
+// searches: one query, top-5, 217 us (lookup scan) -> 162; 32 queries 484 us
+// (k_scan_mma) -> 216; four queries of 1,000 tenants 857 -> 175; eight queries over
+// 250,007 rows 425 -> 79.
 //
 // Two uses:
 //  * BOUND = false, 16 <= nq <= 32: the scores themselves, fp16 products with
@@ -37,9 +38,9 @@
 //
 // Roles (27 warps): 0-15 decoders in four groups of four warps (one warp per
 // TMEM lane quarter; group g takes the 128-coordinate blocks it = g, g + 4,
-// ...; block it goes to TMEM stage it % 6); 16-23 epilogue in two groups (one vector per thread, all
-// queries); 24 code producer (TMA); 25, 26 MMA issuers.  Waits are bounded as in
-// every pipeline here.
+// ...; block it goes to TMEM stage it % 6); 16-23 epilogue in two groups (one
+// vector per thread, all queries); 24 code producer (TMA); 25, 26 MMA issuers.
+// Waits are bounded as in every pipeline here.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -218,7 +219,8 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
 k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict__ qrot,
           const float* __restrict__ centroids, const float* __restrict__ scale, const uint32_t* __restrict__ del,
           const uint32_t* __restrict__ dense, const uint32_t* __restrict__ allow_bits, int words,
-          const uint32_t* __restrict__ bmask, int mask_words, int fblock, const float* __restrict__ bias, int n, int nq, int d, int k, int C, int cst, float* __restrict__ cand_s,
+          const uint32_t* __restrict__ bmask, int mask_words, int fblock, const float* __restrict__ bias, int n,
+          int nq, int d, int k, int C, int cst, float* __restrict__ cand_s,
           int* __restrict__ cand_i, int* __restrict__ err, int* __restrict__ force, uint32_t* __restrict__ gth,
           float* __restrict__ lows) {
   extern __shared__ unsigned char smem_dyn[];
@@ -734,8 +736,9 @@ constexpr int RS_CAP = 1024;  // candidates one block scores
 constexpr int RS_PER = 5;     // list entries per thread: 152 lists of 32
 
 // (The kernel is one short block per query, so its time is latency: few
-// dependent round trips, and rolled loops, since the instructions come from L2
-// too: the unrolled form took 12 us for one query.)
+// dependent round trips, rolled loops, since the instructions come from L2 too
+// (the unrolled form took 12 us for one query), and 32 warps, so that the usual
+// number of candidates is scored in one go (16 warps: 2 us more).)
 __global__ void __launch_bounds__(RS_NT)
 k_rescore(const float* __restrict__ qrot, int d, const float* __restrict__ centroids,
           const uint8_t* __restrict__ codes, const float* __restrict__ scale, int k, int C, int nl,
@@ -761,7 +764,8 @@ k_rescore(const float* __restrict__ qrot, int d, const float* __restrict__ centr
   // one round trip: the force word, the query, every list's two bounds and the lists
   const int forced = __ldcg(force);
   const float bq = bias ? bias[q] : 0.f;
-  if (tid < d / 4) reinterpret_cast<float4*>(sq)[tid] = __ldcg(reinterpret_cast<const float4*>(qrot + (size_t)q * d) + tid);
+  if (tid < d / 4)
+    reinterpret_cast<float4*>(sq)[tid] = __ldcg(reinterpret_cast<const float4*>(qrot + (size_t)q * d) + tid);
   float hl = -INFINITY, kl = -INFINITY;  // of the lists l = lane, lane + 32, ... (every warp alike)
 #pragma unroll 5
   for (int l = lane; l < nl; l += 32) {
@@ -907,7 +911,8 @@ int scan_tm_grid_x(int64_t n) {
 cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* centroids, const uint8_t* codes,
                            const float* scale, int64_t n, const uint32_t* del, const uint32_t* dense,
                            const uint32_t* allow_bits, int words, const uint32_t* bmask, int mask_words, int fblock,
-                           const float* bias, int k, bool bound, float* cand_s, int32_t* cand_i, int* err, int* force, uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
+                           const float* bias, int k, bool bound, float* cand_s, int32_t* cand_i, int* err, int* force,
+                           uint32_t* gth, float* lows, cudaStream_t s, cudaEvent_t ev0,
                            cudaEvent_t ev1) {
   if (nq == 0) return cudaSuccess;
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
@@ -933,7 +938,8 @@ cudaError_t launch_scan_tm(const float* qrot, int64_t nq, int d, const float* ce
     const cudaError_t r = set_max_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)smem);
     if (r != cudaSuccess) return r;
     return launch_maybe_pdl(pdl, kernel, grid, block, smem, s, map, qrot, centroids, scale, del, dense, allow_bits,
-                            words, bmask, mask_words, fblock, bias, (int)n, (int)nq, d, k, C, cst, cand_s, cand_i, err, force, gth, lows);
+                            words, bmask, mask_words, fblock, bias, (int)n, (int)nq, d, k, C, cst, cand_s, cand_i, err,
+                            force, gth, lows);
   };
   e = bound ? (bmask ? go(k_scan_tm<16, true, true>) : go(k_scan_tm<16, true, false>))
             : N == 16 ? go(k_scan_tm<16, false, false>) : go(k_scan_tm<32, false, false>);
