@@ -34,7 +34,7 @@ def _tf32(tq, torch, X, plan, c, t, bits, mode):
 
 
 @pytest.mark.parametrize("n,d,bits,mode", [
-    (1, 1024, 4, "norm"),           # one row, the smallest d
+    (1, 1024, 4, "norm"),           # one row, the smallest d of 4-bit codes
     (129, 1056, 3, "unbiased"),     # a row past a panel; a partial chunk
     (1_000, 1536, 4, "norm"),      # fewer items than SMs
     (2_500, 1536, 8, "none"),      # 20 panels
