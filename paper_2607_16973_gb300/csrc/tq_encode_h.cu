@@ -381,6 +381,11 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
           ok = false;
           break;
         }
+        // The stage's copies were queued after the MMAs of its last use had read
+        // this stage's columns of tensor memory (commit -> empty -> producer ->
+        // full); the fence orders the stores below behind that chain.  (A
+        // wait for `empty` here as well costs a fifth: 12.5 -> 15.2 ms, 999,000 x 1536.)
+        tc_fence_after();
         const unsigned char* xt = base + s * H_STAGE_BYTES + t * 128;
         uint32_t hv[16], lv[16];
 #pragma unroll

@@ -281,6 +281,10 @@ k_encode_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       const long long cs = it / KB;
       const int c = (int)(cs % C), i = (int)(cs / C);
       if (!warp_wait(full + s, (uint32_t)(use & 1), abort_flag, err, 44)) break;
+      // The stage's copies were queued after the MMAs of its last use had read
+      // this stage's columns of tensor memory (commit -> empty -> producer ->
+      // full); the fence orders the stores below behind that chain.
+      tc_fence_after();
       const unsigned char* xt = base + s * ENC_STAGE_BYTES;
       float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
       uint32_t hv[EK], lv[EK];  // row t's x_hi and x_lo, in K order
