@@ -297,7 +297,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
   const int nqt = (nq + MMA_M - 1) / MMA_M;
   const int qts = min(QT, nqt - qt0);                  // query tiles present (1..QT)
   const int kblocks = d / KB;
-  const int ntiles = (n + NT - 1) / NT;
+  const int ntiles = row_tiles(n, NT);
   const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (BITS == 2) {

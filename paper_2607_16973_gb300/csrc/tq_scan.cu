@@ -392,7 +392,7 @@ k_scan_stream(const float* __restrict__ qrot, int d, const float* __restrict__ c
   int cnt = 0;
   float th_s = -INFINITY;
   int th_i = INT_MAX;
-  const int nsteps = (n + SCAN_WARPS * V - 1) / (SCAN_WARPS * V);
+  const int nsteps = row_tiles(n, SCAN_WARPS * V);
   const int my = (lane >> 3) & 3;  // the vector whose total this lane ends up holding
   const uint32_t lane4 = (uint32_t)lane * 4u;
   const char* tab = reinterpret_cast<const char*>(smem_raw);
@@ -585,7 +585,8 @@ k_scan_ring(const float* __restrict__ qrot, int d, const float* __restrict__ cen
   __shared__ volatile int abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = blockIdx.y;
-  const int nsteps = (n + V - 1) / V;  // warp steps of 4 vectors
+  const int nsteps = row_tiles(n, V);  // warp steps of 4 vectors
+  const int whole = n / V;             // of them whole ones
   const int wstride = gridDim.x * RING_WARPS;
   uint64_t* wbar = bars + warp * RING_MAX_NS;
   unsigned char* wring = ring + (size_t)warp * ns * slot_bytes;
@@ -606,7 +607,7 @@ k_scan_ring(const float* __restrict__ qrot, int d, const float* __restrict__ cen
     __syncwarp();  // every lane has read the slot's previous codes
     if (lane == 0) {
       stepq[warp][s] = ws;
-      if (ws < nsteps && (ws + 1) * V <= n) {
+      if (ws < whole) {
         ring_copy(wring + s * slot_bytes, codes + (size_t)ws * slot_bytes, (uint32_t)slot_bytes, wbar + s);
         pend |= 1u << s;
       }
@@ -676,7 +677,7 @@ k_scan_ring(const float* __restrict__ qrot, int d, const float* __restrict__ cen
     if (abort_flag) break;
     const int v0 = ws * V;
     Chunk<BITS> cur[V][S];
-    if (v0 + V <= n) {  // whole step: its codes came by bulk copy
+    if (ws < whole) {  // whole step: its codes came by bulk copy
       bool ok = true;
       if (lane == 0) ok = bounded_wait(wbar + s, (par >> s) & 1u, &abort_flag, err, 20, kWaitCycles);
       ok = __shfl_sync(FULL, ok ? 1 : 0, 0) != 0;

@@ -248,7 +248,7 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
   auto gapw = [&](int w) { return lut + ((uint32_t)w >> 5) * 256u + 128u + ((uint32_t)w & 31u) * 4u; };
 
   const int tid = threadIdx.x, warp = __shfl_sync(FULL, tid >> 5, 0), lane = tid & 31;
-  const int ntiles = (n + TM_M - 1) / TM_M;
+  const int ntiles = row_tiles(n, TM_M);
   const int all_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int raws = d >> 8;        // raw code tiles per vector tile
   const int blks = d / TM_BLK;    // decoded blocks per vector tile
