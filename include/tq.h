@@ -260,7 +260,10 @@ tq_status tq_filter_info(const tq_filter* filter, int64_t* n, int* block,
 /*
  * tq_search_workspace - bytes of device scratch tq_search needs for these
  * sizes on the current device (query rotation, allow bitmaps, per-CTA top-k
- * candidates).  filter may be NULL (unfiltered).
+ * candidates).  filter may be NULL (unfiltered).  The bytes are enough for
+ * every search of up to nq queries and up to k results over the same n, d and
+ * bits, with the filter or without one: a workspace kept for a program's
+ * largest search serves its smaller ones.
  */
 tq_status tq_search_workspace(int64_t nq, int64_t n, int d, int bits, int k,
                               const tq_filter* filter, size_t* bytes);

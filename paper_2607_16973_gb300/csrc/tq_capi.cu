@@ -51,8 +51,9 @@ SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_f
   const bool tm = scan_tm_supported(nq, n, d, bits, k, true, filter != nullptr);
   const bool tm16 = scan_tm_supported(nq, n, d, bits, k, false, filter != nullptr);
   p.grid_tm = tm || tm16 ? scan_tm_grid_x(n) : 0;
-  const int per_query = std::max(std::max(std::max(p.grid_lut, p.grid_mma), p.grid_fold) * k,
-                                 p.grid_tm * scan_tm_list(k, tm));
+  const int64_t per_query = std::max(std::max(std::max(p.grid_lut, p.grid_mma), p.grid_fold) * k,
+                                     p.grid_tm * scan_tm_list(k, tm));
+  const size_t cand = (size_t)std::max(nq * per_query, scan_lut_max_lists(nq, n, k, bits, d) * k);
   size_t off = 0;
   p.off_status = off;
   off = align_up(off + sizeof(int));
@@ -79,11 +80,40 @@ SearchPlan plan_search(int64_t nq, int64_t n, int d, int bits, int k, const tq_f
   p.off_lists = off;
   if (mma) off = align_up(off + mma_list_bytes(nq, bits, k, p.grid_mma));
   p.off_cs = off;
-  off = align_up(off + (size_t)nq * per_query * sizeof(float));
+  off = align_up(off + cand * sizeof(float));
   p.off_ci = off;
-  off = align_up(off + (size_t)nq * per_query * sizeof(int32_t));
+  off = align_up(off + cand * sizeof(int32_t));
   p.total = off;
   return p;
+}
+
+// Bytes that serve every search of up to nq queries and up to k results, with
+// the filter or without, so that a workspace kept for a program's largest
+// search is enough for its smaller ones.  The layout grows with nq, k and the
+// filter except where the larger search takes another path or splits its work
+// less: behind the exact small-batch search (less than kMmaMinBatch queries,
+// k <= 16 or 32, see scan_tm_supported), behind the small-batch scan, behind
+// the batched scan's largest k, and at each query tile (rotation splits; CTAs
+// per group of tiles, until there is one).
+size_t search_bytes(int64_t nq, int64_t n, int d, int bits, int k, const tq_filter* filter) {
+  size_t need = 0;
+  auto also = [&](int64_t m, int kk, const tq_filter* f) {
+    need = std::max(need, plan_search(m, n, d, bits, kk, f).total);
+  };
+  const int ks[4] = {k, std::min(k, kMaxKMma), std::min(k, kTmMaxK), std::min(k, kTmSmallK)};
+  for (int i = 0; i < 4; ++i) {
+    if (i && ks[i] == ks[i - 1]) continue;
+    also(nq, ks[i], filter);
+    const int64_t small[2] = {std::min<int64_t>(nq, kMmaMinBatch - 1), std::min<int64_t>(nq, kTmMaxBatch)};
+    for (const int64_t m : small) {
+      also(m, ks[i], filter);
+      if (filter) also(m, ks[i], nullptr);
+    }
+    if (i > 1) continue;  // (of the batched scan's searches the largest k needs most)
+    const int64_t last = std::min(nq - 1, (int64_t)2 * kQueryTile * device_sm_count());
+    for (int64_t m = kQueryTile; m <= last; m += kQueryTile) also(m, ks[i], filter);
+  }
+  return need;
 }
 
 }  // namespace
@@ -446,7 +476,7 @@ extern "C" tq_status tq_search_workspace(int64_t nq, int64_t n, int d, int bits,
   if (!bytes) return fail(TQ_EINVAL, "tq_search_workspace: NULL bytes");
   tq_status st = check_search(nq, n, d, bits, k);
   if (st != TQ_OK) return st;
-  *bytes = tq::plan_search(nq, n, d, bits, k, filter).total;
+  *bytes = tq::search_bytes(nq, n, d, bits, k, filter);
   return tq::ok();
 }
 

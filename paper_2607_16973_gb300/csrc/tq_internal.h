@@ -24,6 +24,10 @@ constexpr int kMaxKMma = 64;     // per-thread top-k lists of the tensor-core sc
 constexpr int kMmaMinBatch = 16; // AUTO uses the tensor-core scan from this batch size
 constexpr int kMaxD = 8192;
 constexpr int kRotTcMinBatch = 16;  // query batches rotated on the tensor cores from this size
+constexpr int kTmMaxBatch = 32;   // queries of the small-batch tensor-core scan
+constexpr int kTmMaxK = 32;       // its largest k, and the k up to which fewer rows are enough for the exact search
+constexpr int kTmSmallK = 16;
+constexpr int kQueryTile = 128;   // queries per tile of the batched scan and the tensor-core rotation
 constexpr int kTmMinRows = 2048;  // the exact tensor-core search of small batches needs this many rows
 // The fixed-point 4-bit centroid table (TQ_PATH_LUT_FIXED) applies from this
 // d on: its rounding error is about 2^-16 of the largest centroid (~3.5 /

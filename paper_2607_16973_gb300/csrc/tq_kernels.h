@@ -95,6 +95,7 @@ cudaError_t launch_filter_raw_ids(const FilterDev& f, uint32_t* raw, cudaStream_
 // per-query term, added to each raw score before the per-vector scale.  `gate`
 // [nq] (nullable; not for 3-bit codes): only queries with gate[q] != 0 are searched.
 int scan_lut_grid_x(int64_t nq, int64_t n, int k, int bits, int d);
+int64_t scan_lut_max_lists(int64_t nq, int64_t n, int k, int bits, int d);  // of any batch of up to nq queries
 cudaError_t launch_scan_lut(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
                             const uint8_t* codes, const float* scale, int64_t n, const uint32_t* del,
                             const FilterDev* f, const uint32_t* allow_bits, const uint32_t* bmask, bool fix,
@@ -148,7 +149,7 @@ cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* c
                             uint32_t* heads, uint64_t* lists, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1);
 
 // Small-batch tensor-core scan of 4-bit codes (k_scan_tm).  With `bound` it is
-// the first half of an exact float32 search of at most 16 queries: every CTA
+// the first half of an exact float32 search of fewer than 16 queries: every CTA
 // keeps the scan_tm_list(k, true) vectors whose upper score bounds are best,
 // and launch_rescore scores the candidates as the lookup scan does, writes the
 // results and sets gate[q] for the queries it could not settle (the lookup

@@ -1072,10 +1072,20 @@ cudaError_t scan_bits(int S, bool filt, bool fix, dim3 grid, size_t smem, cudaSt
 
 }  // namespace
 
+// One resident wave for a single query: one ring-scan CTA per SM, or two
+// register-fed CTAs.
+static int64_t lut_wave(int bits, int d, int k) {
+  return (int64_t)device_sm_count() * (ring_slots(bits, d, k) >= 2 ? 1 : 2);
+}
+
+// m * scan_lut_grid_x(m) for m <= nq is at most a wave and m - 1, and at most
+// one list per 32 rows and query.
+int64_t scan_lut_max_lists(int64_t nq, int64_t n, int k, int bits, int d) {
+  return nq < 1 ? 0 : std::min(nq * ((n + 31) / 32), lut_wave(bits, d, k) + nq - 1);
+}
+
 int scan_lut_grid_x(int64_t nq, int64_t n, int k, int bits, int d) {
-  // one resident wave for a single query: one ring-scan CTA per SM, or two
-  // register-fed CTAs
-  const int64_t target = (int64_t)device_sm_count() * (ring_slots(bits, d, k) >= 2 ? 1 : 2);
+  const int64_t target = lut_wave(bits, d, k);
   int64_t gx = (target + nq - 1) / (nq > 0 ? nq : 1);
   const int64_t blocks = (n + 31) / 32;
   if (gx > blocks) gx = blocks;

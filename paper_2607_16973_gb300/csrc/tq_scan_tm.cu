@@ -25,7 +25,7 @@
 // Two uses:
 //  * BOUND = false, 16 <= nq <= 32: the scores themselves, fp16 products with
 //    float32 accumulation, the same operand rounding as k_scan_mma.
-//  * BOUND = true, nq <= 16: an exact float32 search.  The scan computes, per
+//  * BOUND = true, nq < 16: an exact float32 search.  The scan computes, per
 //    vector, an upper bound U of the score the lookup scan would give: the
 //    fp16 score plus a bound of everything it leaves out (the rounding of both
 //    operands, summed exactly per query and codebook, and the accumulation
@@ -76,7 +76,7 @@ constexpr uint32_t TM_SMEM_MAX = 232448;  // 227 KB per block
 // hold two tiles' candidate scores (and with 16 columns 2 * 128 their |scale|).
 constexpr int TM_TILE_LIST = 2 * 16 * TM_M + 2 * TM_M;  // first word of the tile list (16 columns)
 constexpr int TM_MAX_TILES = 8192 - TM_TILE_LIST;
-constexpr int TM_LIST = 32;               // entries of a query's list in a CTA (one per lane)
+constexpr int TM_LIST = kTmMaxK;          // entries of a query's list in a CTA (one per lane)
 constexpr uint32_t TM_A_COL = 128;        // TMEM: two sets of two accumulators of N <= 32 columns, then the stages
 // misc area (after the raw tiles): per-query values, masks, barriers
 struct TmMisc {
@@ -895,11 +895,12 @@ k_rescore(const float* __restrict__ qrot, int d, const float* __restrict__ centr
 // tiles are read once for all of them.
 bool scan_tm_supported(int64_t nq, int64_t n, int d, int bits, int k, bool bound, bool filtered) {
   if (bits != 4 || d % 256 != 0 || d > 2048 || k > TM_LIST || nq < 1) return false;
+  if (bound && nq >= kMmaMinBatch) return false;
   if (filtered && bound)
-    return nq >= 2 && nq <= 16 && n * d * nq >= (int64_t)1 << 26 &&
+    return nq >= 2 && n * d * nq >= (int64_t)1 << 26 &&
            (n + TM_M - 1) / TM_M <= (int64_t)TM_MAX_TILES * device_sm_count();
-  if (bound) return nq <= 16 && n >= kTmMinRows && n * d * nq >= (k <= 16 ? (int64_t)1 << 24 : (int64_t)1 << 27);
-  return nq <= 32;
+  if (bound) return n >= kTmMinRows && n * d * nq >= (k <= kTmSmallK ? (int64_t)1 << 24 : (int64_t)1 << 27);
+  return nq <= kTmMaxBatch;
 }
 
 int scan_tm_list(int k, bool bound) { return bound ? TM_LIST : k; }
