@@ -102,8 +102,10 @@ def encode(X, R, centroids, boundaries, bits: int, scale_mode: str = "norm",
     scale f32 [n]).  With `plan` (encode_plan(R)) the rotation runs on the
     tensor cores (tq_encode_planned_ws) and R is not read; `workspace`
     (CUDA uint8, encode_workspace(n, d) bytes) may be kept between calls,
-    otherwise one is allocated, or, where it does not fit in device memory, the
-    encoder that needs none runs (tq_encode_planned)."""
+    otherwise one is allocated, and a failure to allocate it is raised: the
+    encoder that needs none decides some coordinates next to a cell boundary
+    differently, so it runs only where it is asked for, with
+    `workspace=False` (tq_encode_planned), or where no workspace is read."""
     torch = _torch()
     n, d = X.shape
     with _on_stream(stream):
@@ -121,13 +123,10 @@ def encode(X, R, centroids, boundaries, bits: int, scale_mode: str = "norm",
         # below these d the fp16 encoder does not run and reads no workspace
         need = encode_workspace(n, d) if d >= (768 if bits == 8 else 1024) else None
         if workspace is None and need is not None:
-            try:
-                with _on_stream(stream):
-                    workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
-            except torch.OutOfMemoryError:
-                pass
+            with _on_stream(stream):
+                workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
         head = (_dev_ptr(X, "X", f32), n, d, _dev_ptr(plan, "plan", torch.uint8))
-        if workspace is not None:
+        if workspace is not None and workspace is not False:
             check(load().tq_encode_planned_ws(*head, *tail, _dev_ptr(workspace, "workspace"),
                                               workspace.numel() * workspace.element_size(), handle))
         else:

@@ -109,6 +109,29 @@ def test_encode_h_workspace(cuda_lib, tdev):
     assert tq.encode_workspace(n, 96) is None
 
 
+def test_no_memory_for_the_workspace(cuda_lib, tdev, monkeypatch):
+    """The encoder is the caller's choice, not the free memory's: a workspace
+    that cannot be allocated is an error; without one on request, the codes are
+    the TF32 encoder's."""
+    torch, dev, T = tdev
+    tq = cuda_lib
+    n, d, bits = 300, 1024, 4
+    c, t = (T(a) for a in _cb(d, bits))
+    X, plan = T(synth.gaussian_rows(n, d, seed=9)), tq.encode_plan(T(O.rotation(d, 7).astype(np.float32)))
+    out = torch.empty((n, d * bits // 8), dtype=torch.uint8, device=dev), torch.empty(n, device=dev)
+
+    def no_memory(*a, **kw):
+        raise torch.OutOfMemoryError("no memory")
+
+    with monkeypatch.context() as m:
+        m.setattr(torch, "empty", no_memory)
+        with pytest.raises(torch.OutOfMemoryError):
+            tq.encode(X, None, c, t, bits, "norm", *out, plan=plan)
+        codes, scale = tq.encode(X, None, c, t, bits, "norm", *out, plan=plan, workspace=False)
+    codes_t, scale_t = _tf32(tq, torch, X, plan, c, t, bits, "norm")
+    assert np.array_equal(codes.cpu().numpy(), codes_t) and np.array_equal(scale.cpu().numpy(), scale_t)
+
+
 @pytest.mark.parametrize("d,bits", [(384, 3), (992, 4), (736, 8)])
 def test_below_its_range_the_tf32_encoder_runs(cuda_lib, tdev, d, bits):
     torch, dev, T = tdev
