@@ -203,6 +203,8 @@ tq_status tq_encode_ex(const float* X, int64_t n, int d, const float* R,
  *                tq_encode_planned and reads no workspace.)  The
  *                workspace is free again when the call's work has finished.
  *                n up to 2^31 - 1024.
+ * tq_encode_workspace_for  the same for one code width: 0 where
+ *                tq_encode_planned_ws reads no workspace at that d and bits.
  */
 tq_status tq_encode_plan_bytes(int d, size_t* bytes);
 tq_status tq_encode_plan(const float* R, int d, void* plan, size_t plan_bytes, void* stream);
@@ -211,6 +213,7 @@ tq_status tq_encode_planned(const float* X, int64_t n, int d, const void* plan,
                             int scale_mode, const float* cal_mu, const float* cal_a,
                             uint8_t* codes, float* scale, void* stream);
 tq_status tq_encode_workspace(int64_t n, int d, size_t* bytes);
+tq_status tq_encode_workspace_for(int64_t n, int d, int bits, size_t* bytes);
 tq_status tq_encode_planned_ws(const float* X, int64_t n, int d, const void* plan,
                                const float* centroids, const float* boundaries, int bits,
                                int scale_mode, const float* cal_mu, const float* cal_a,

@@ -120,9 +120,8 @@ def encode(X, R, centroids, boundaries, bits: int, scale_mode: str = "norm",
             _dev_ptr(codes, "codes", torch.uint8), _dev_ptr(scale, "scale", f32))
     handle = _stream_handle(stream)
     if plan is not None:
-        # below these d the fp16 encoder does not run and reads no workspace
-        need = encode_workspace(n, d) if d >= (768 if bits == 8 else 1024) else None
-        if workspace is None and need is not None:
+        need = encode_workspace(n, d, bits) if workspace is None else None
+        if need:
             with _on_stream(stream):
                 workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
         head = (_dev_ptr(X, "X", f32), n, d, _dev_ptr(plan, "plan", torch.uint8))
@@ -147,12 +146,16 @@ def encode_plan_bytes(d: int):
     return need.value
 
 
-def encode_workspace(n: int, d: int):
+def encode_workspace(n: int, d: int, bits: int | None = None):
     """tq_encode_workspace: device bytes of scratch for encoding n rows with a
-    plan, or None where that encoder does not apply."""
+    plan, or None where that encoder does not apply.  With `bits`
+    (tq_encode_workspace_for) 0 where it reads none at that width."""
     need = C.c_size_t()
     try:
-        check(load().tq_encode_workspace(n, d, C.byref(need)))
+        if bits is None:
+            check(load().tq_encode_workspace(n, d, C.byref(need)))
+        else:
+            check(load().tq_encode_workspace_for(n, d, bits, C.byref(need)))
     except TQError:
         return None
     return need.value

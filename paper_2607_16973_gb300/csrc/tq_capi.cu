@@ -226,6 +226,14 @@ extern "C" tq_status tq_encode_workspace(int64_t n, int d, size_t* bytes) {
   return tq::ok();
 }
 
+extern "C" tq_status tq_encode_workspace_for(int64_t n, int d, int bits, size_t* bytes) {
+  const tq_status st = tq_encode_workspace(n, d, bytes);
+  if (st != TQ_OK) return st;
+  if (!tq::valid_bits(bits)) return fail(TQ_EINVAL, "tq_encode_workspace_for: bits=%d must be 2, 3, 4 or 8", bits);
+  if (!tq::encode_h_applies(d, bits)) *bytes = 0;
+  return tq::ok();
+}
+
 extern "C" tq_status tq_encode_planned_ws(const float* X, int64_t n, int d, const void* plan,
                                           const float* centroids, const float* boundaries, int bits,
                                           int scale_mode, const float* cal_mu, const float* cal_a, uint8_t* codes,

@@ -213,3 +213,15 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(_lib, "LIB_PATH", str(tmp_path / "libtq.so"))
     with pytest.raises(RuntimeError, match="missing"):
         _lib.load()
+
+
+def test_encode_workspace_by_width(lib):
+    """Where the planned encoder reads a workspace: from d = 1024 on, 8-bit
+    codes from 768; the answer comes from the library's own rule."""
+    for d, bits, reads in [(992, 4, False), (1024, 4, True), (1024, 2, True), (736, 8, False), (768, 8, True),
+                           (992, 3, False)]:
+        assert tq.encode_workspace(1000, d, bits) == (tq.encode_workspace(1000, d) if reads else 0), (d, bits)
+    assert tq.encode_workspace(1000, 96, 4) is None and tq.encode_workspace(1000, 96) is None
+    sz = C.c_size_t()
+    assert lib.tq_encode_workspace_for(1000, 1024, 5, C.byref(sz)) == _lib.TQ_EINVAL
+    assert lib.tq_encode_workspace_for(1000, 1024, 4, None) == _lib.TQ_EINVAL
