@@ -498,9 +498,11 @@ tq_status tq_debug_bounded_wait(long long budget_cycles, void* workspace,
 tq_status tq_set_search_path(int path);
 
 /* Records two caller-created CUDA events (cudaEvent_t passed as void*) on the
- * search stream immediately before and after the scan kernel of the calling
- * thread's later tq_search calls, for per-kernel timing.  NULL, NULL turns it
- * off. */
+ * search stream immediately before and after the scan of the calling thread's
+ * later tq_search calls, for per-kernel timing: one kernel, or for the exact
+ * small-batch search the bounding scan, the rescoring and the lookup scan
+ * behind its gates, which together do what the lookup scan does alone.  NULL,
+ * NULL turns it off. */
 tq_status tq_profile_events(void* scan_start, void* scan_stop);
 
 #ifdef __cplusplus

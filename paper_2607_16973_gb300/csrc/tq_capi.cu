@@ -568,16 +568,17 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
       e = tq::launch_scan_tm(qrot, nq, d, centroids, codes, scale, n, deleted, filter ? filter->f.dense : nullptr,
                              allow, filter ? filter->f.words : 0, tm_bound ? bmask : nullptr,
                              filter ? tq::filter_mask_words(filter->f) : 0, filter ? filter->f.block : 64, bias, k,
-                             tm_bound, cs, ci, status, force, gth, lows, s,
-                             (cudaEvent_t)tq::profile_start(), (cudaEvent_t)tq::profile_stop());
+                             tm_bound, cs, ci, status, force, gth, lows, s, (cudaEvent_t)tq::profile_start(),
+                             tm_bound ? nullptr : (cudaEvent_t)tq::profile_stop());
     if (tm_bound) {
       if (e == cudaSuccess)
         e = tq::launch_rescore(qrot, nq, d, centroids, codes, scale, n, k, cs, ci, lows, force, gate, ext_ids, out_ids,
                                out_scores, bias, s);
       if (e == cudaSuccess)
         e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
-                                filter ? &filter->f : nullptr, allow, bmask, false, k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias,
-                                gate, s, nullptr, nullptr);
+                                filter ? &filter->f : nullptr, allow, bmask, false, k, p.grid_lut, cs, ci, status,
+                                counters, ext_ids, out_ids, out_scores, bias, gate, s, nullptr,
+                                (cudaEvent_t)tq::profile_stop());
     } else if (e == cudaSuccess) {
       e = tq::launch_merge(cs, ci, nq, p.grid_tm * k, k, ext_ids, out_ids, out_scores, s);
     }

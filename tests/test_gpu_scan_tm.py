@@ -198,3 +198,28 @@ def test_exact_search_filtered(cuda_lib, tdev, order, block):
     allowed = np.stack([np.isin(tenants, v) for v in lists])
     ref = O.search(Q, R, c32, 4, packed, scale, k, d, tenant_ids=tenants, allow_off=off, allow_ids=ten)
     check_topk(ids, sc, ref.ids, ref.scores64, allowed, k, TOL_LUT)
+
+
+def test_profile_events_cover_the_whole_exact_scan(cuda_lib, tdev):
+    """The events stand around the bounding scan, the rescoring and the gated
+    lookup scan.  One scale the bounds do not cover opens the gate, so between
+    them lies more than the lookup scan alone takes."""
+    torch, T = tdev
+    tq = cuda_lib
+    d, n = 1536, 200_000
+    packed, scale, R, Q = _data(n, d, 1, seed=51)
+    scale[100] = np.nan
+    a = (T(Q), T(R), T(_cb(d)[0]), 4, T(packed), T(scale), 10)
+    ms = {}
+    for path in ("lut", "auto"):
+        times = []
+        for _ in range(7):
+            ev = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            tq.profile_events(*ev)
+            try:
+                _search(tq, torch, path, *a)
+            finally:
+                tq.profile_events(None, None)
+            times.append(ev[0].elapsed_time(ev[1]))
+        ms[path] = sorted(times)[3]
+    assert ms["auto"] > 1.3 * ms["lut"], ms
