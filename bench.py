@@ -70,7 +70,6 @@ CONFIGS = {
 }
 
 RECALL_Q = 200       # queries whose Recall@k against exact kNN the bench reports
-MMA_MIN_BATCH = 16  # tq_search's AUTO switch to the tensor-core scan (k <= 64)
 
 METRIC = "queries/sec at 999Kx1536 4-bit top-5 (batch 1 / 1024); % of HBM / TC roofline"
 
@@ -100,23 +99,9 @@ def source_hash(*files):
     return h.hexdigest()[:16]
 
 
-def small_batch_kernel(bits: int, n: int, d: int, k: int, nq: int = 1, path: str = "auto") -> str:
-    """The scan tq_search runs for an unfiltered batch below 16 queries: the
-    small-batch tensor-core scan (exact: its candidates are rescored in float32)
-    for 4-bit codes and enough work, else a lookup scan: the bulk-copy ring for
-    3-bit codes, the register-fed byte-pair (4-bit) or per-code scan otherwise."""
-    if path == "lut_fold":
-        return "k_scan_fold"
-    if path == "auto" and bits == 4 and d % 256 == 0 and d <= 2048 and k <= 32 and n >= 2048 and \
-            n * d * nq >= (1 << 24 if k <= 16 else 1 << 27):
-        return "k_scan_tm"
-    return "k_scan_ring" if bits == 3 else "k_scan_stream"
-
-
-def fp16_kernel(bits: int, d: int, k: int, nq: int, path: str = "auto") -> str:
-    """The tensor-core scan of a batch of 16 or more queries."""
-    small = path == "auto" and nq <= 32 and bits == 4 and d % 256 == 0 and d <= 2048 and k <= 32
-    return "k_scan_tm" if small else "k_scan_mma"
+TENSOR_SCANS = ("k_scan_mma", "k_scan_tm")  # of tq.search_kernel's: fp16 products, against the tensor peak
+# kernels behind the rotation: packing + scan + merge; scan + merge; bounding scan + rescoring + gated lookup scan
+SCAN_LAUNCHES = {"k_scan_mma": 3, "k_scan_tm": 2, "k_scan_tm (exact)": 3}
 
 
 def recorded_traffic(kernel_file, profile_md: str, scale_to: int):
@@ -477,9 +462,8 @@ def run_ours(args, cfg, rank, world):
         scan_ms = statistics.mean(a.elapsed_time(b) for a, b in evs)
         qps = B * args.steps * world / (ms / 1e3)
         alg_bytes = n * (d * bits // 8 + 4)
-        mma = bits in (2, 4, 8, 3) and k <= 64 and (args.search_path == "mma" or
-                                                    (args.search_path == "auto" and B >= MMA_MIN_BATCH))
-        if mma:
+        kern = tq.search_kernel(B, n, d, bits, k)  # on --search-path
+        if kern in TENSOR_SCANS:
             # tensor-core scan: 2*n*d*B flops per launch against the dense fp16/bf16
             # peak (same rate); each launch is a few ms, timed alone: the burst figure
             flops = 2.0 * n * d * B
@@ -490,14 +474,13 @@ def run_ours(args, cfg, rank, world):
                     "frac_of_sustained": achieved / pk["bf16_tflops_sustained"],
                     "traffic": recorded_traffic("paper_2607_16973_gb300/csrc/tq_mma.cu", "k_scan_mma_250k_batch1024.md",
                                                 scale_to=n) if B >= 1024 else None,
-                    "kernel": fp16_kernel(bits, d, k, B, args.search_path), "alg_flops_per_launch": flops, "kernel_ms": scan_ms,
+                    "kernel": kern, "alg_flops_per_launch": flops, "kernel_ms": scan_ms,
                     "hbm_gbs_of_corpus": alg_bytes / (scan_ms / 1e3) / 1e9}
         else:
-            # lookup scan (with its last CTA's merge): the corpus, codes + scales,
-            # read once per launch
+            # lookup scan (with its last CTA's merge), or the bounding scan with its
+            # rescoring: the corpus, codes + scales, read once
             achieved = alg_bytes / (scan_ms / 1e3) / 1e9
-            kern = small_batch_kernel(bits, n, d, k, B, args.search_path)
-            if kern == "k_scan_tm":
+            if kern == "k_scan_tm (exact)":
                 traffic = recorded_traffic("paper_2607_16973_gb300/csrc/tq_scan_tm.cu", "k_scan_tm_250k_batch1.md",
                                            scale_to=n)
             elif kern == "k_scan_fold":
@@ -547,10 +530,8 @@ def run_ours(args, cfg, rank, world):
         e2e_ms = a.elapsed_time(b)
         # our kernels per step: the rotation (with its reduce from 16 queries on:
         # the tensor-core rotation), then the lookup scan (merged in its last
-        # CTA), or the bounding scan + rescoring + the lookup scan behind its
-        # gates, or (query packing +) tensor-core scan + merge; + the shard merge
-        scan_launches = {"k_scan_mma": 3, "k_scan_tm": 2 if mma else 3}.get(roof["kernel"], 1)
-        launches = (2 if B >= 16 else 1) + scan_launches + (1 if world > 1 else 0)
+        # CTA) or SCAN_LAUNCHES; + the shard merge
+        launches = (2 if B >= 16 else 1) + SCAN_LAUNCHES.get(kern, 1) + (1 if world > 1 else 0)
         results[B] = {
             "value": qps, "ms_per_step": ms / args.steps, "roofline": roof, "clocks": clk.summary(),
             "gpu_launches": launches * args.steps,
@@ -712,11 +693,11 @@ def _roof_hbm(alg_bytes, ms, pk, kernel):
             "kernel_ms": ms}
 
 
-def _roof_tc(flops, ms, pk):
+def _roof_tc(flops, ms, pk, kernel):
     tf = flops / (ms / 1e3) / 1e12
     return {"bound": "tensor", "achieved": tf, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
             "frac": tf / pk["bf16_tflops"], "frac_of": pk["source"] + " burst bf16 (= fp16 dense rate)",
-            "traffic": None, "kernel": "k_scan_mma", "alg_flops_per_launch": flops, "kernel_ms": ms}
+            "traffic": None, "kernel": kernel, "alg_flops_per_launch": flops, "kernel_ms": ms}
 
 
 def _roof_encode(n, d, ms, pk):
@@ -785,15 +766,15 @@ def extras_100k(torch, tq, dev, stream, pk, flush, steps):
                     fn(i)
                 ms = _flushed_ms(torch, fn, steps, stream, flush)
                 kms = _scan_ms(torch, tq, fn, steps, stream, flush)
-                tq.set_search_path("lut" if B < MMA_MIN_BATCH else "auto")
+                tq.set_search_path("lut" if tq.search_kernel(B, n, d, bits, k) not in TENSOR_SCANS else "auto")
                 try:
                     got, _ = tq.search(Qd[:nrec], Rd, cd, bits, codes, scale, k, stream=stream)
                 finally:
                     tq.set_search_path("auto")
                 ex = torch.topk(exact_sc, k, dim=1)[1]
             stream.synchronize()
-            roof = _roof_tc(2.0 * n * d * B, kms, pk) if B >= MMA_MIN_BATCH else _roof_hbm(
-                alg, kms, pk, small_batch_kernel(bits, n, d, k, B))
+            kern = tq.search_kernel(B, n, d, bits, k)
+            roof = _roof_tc(2.0 * n * d * B, kms, pk, kern) if kern in TENSOR_SCANS else _roof_hbm(alg, kms, pk, kern)
             out[f"batch{B}_top{k}"] = {"value": B / ms * 1e3, "unit": "queries/s", "ms_per_step": ms,
                                        "roofline": roof, "recall": _recall(torch, got.cpu(), ex.cpu())}
             log(f"[bench] 100K batch {B} top-{k}: {B / ms * 1e3:.4g} q/s, scan {kms * 1e3:.1f} us")
@@ -858,7 +839,8 @@ def extras_100k(torch, tq, dev, stream, pk, flush, steps):
         live = (1.0 - float(np.mean(skip))) * alg + n * 4  # codes + scales of the blocks read, dense tenant ids
         filt_out[str(T)] = {"value": 1e3 / ms, "unit": "queries/s", "ms_per_query": ms,
                             "bytes_skipped_frac": float(np.mean(skip)), "recall": hits / nrec,
-                            "roofline": _roof_hbm(live, kms, pk, "k_scan_stream (filtered)"),
+                            "roofline": _roof_hbm(live, kms, pk,
+                                                  tq.search_kernel(1, n, d, bits, k, filtered=True) + " (filtered)"),
                             "postfilter": {"overfetch_k": k_over, "recall": pf_hits / nrec, "ms_per_query": ms_over}}
         log(f"[bench] filtered T={T}: {1e3 / ms:.4g} q/s, scan {kms * 1e3:.1f} us, {np.mean(skip):.1%} skipped, "
             f"R@{k} {hits / nrec:.3f}, post-filter R@{k} {pf_hits / nrec:.3f}")
@@ -907,9 +889,10 @@ def extras_sweep(torch, tq, dev, stream, pk, Xd, Rd, Qd, steps):
                           stream=stream)
             ms = _timed(fn, steps, 2, stream)
             kms = _scan_ms(torch, tq, fn, min(steps, 5), stream)
-        mma = bits in (2, 3, 4, 8)
+        kern = tq.search_kernel(B, n, d, bits, k)
+        mma = kern in TENSOR_SCANS
         alg = n * (d * bits // 8 + 4)
-        roof = _roof_tc(2.0 * n * d * B, kms, pk) if mma else _roof_hbm(alg, kms, pk, "k_scan_ring")
+        roof = _roof_tc(2.0 * n * d * B, kms, pk, kern) if mma else _roof_hbm(alg, kms, pk, kern)
         out["variants"][str(bits)] = {"value": B / ms * 1e3, "unit": "queries/s", "ms_per_step": ms,
                                       "path": "tensor core" if mma else "lookup", "roofline": roof,
                                       "encode": {"value": n / enc_ms * 1e3, "unit": "vectors/s", "ms": enc_ms,

@@ -505,6 +505,14 @@ tq_status tq_set_search_path(int path);
  * NULL turns it off. */
 tq_status tq_profile_events(void* scan_start, void* scan_stop);
 
+/* The scan that tq_search takes for these sizes (filtered: with a filter or not)
+ * on the calling thread's path, which tq_profile_events' events stand around:
+ * "k_scan_stream", "k_scan_ring", "k_scan_fold", "k_scan_mma", "k_scan_tm"
+ * (fp16) or "k_scan_tm (exact)" (with its rescoring).  The name is static.
+ * Errors as tq_search's for the same sizes. */
+tq_status tq_search_kernel(int64_t nq, int64_t n, int d, int bits, int k,
+                           int filtered, const char** name);
+
 #ifdef __cplusplus
 }
 #endif

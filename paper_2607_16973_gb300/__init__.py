@@ -15,7 +15,7 @@ from ._lib import (MARGINALS, PATHS, SCALE_MODES, TQ_EUNSUPPORTED, TQError, chec
 
 __all__ = ["codebook", "rotation", "encode", "encode_plan", "encode_plan_bytes", "encode_workspace", "encode_check", "calibrate", "Filter", "IdMap", "Index", "search", "search_workspace",
            "search_from_host", "search_host_staging", "search_check", "merge_topk", "set_search_path",
-           "profile_events", "row_bytes", "load", "TQError"]
+           "profile_events", "search_kernel", "row_bytes", "load", "TQError"]
 
 
 def _torch():
@@ -444,6 +444,14 @@ def search_check(workspace, stream=None) -> None:
 def set_search_path(path: str) -> None:
     """'auto' (default), 'lut' or 'mma' for later searches on this thread."""
     check(load().tq_set_search_path(PATHS[path]))
+
+
+def search_kernel(nq: int, n: int, d: int, bits: int, k: int, filtered: bool = False) -> str:
+    """tq_search_kernel: the scan that a search of these sizes takes on this
+    thread's path, which profile_events' events stand around."""
+    name = C.c_char_p()
+    check(load().tq_search_kernel(nq, n, d, bits, k, int(filtered), C.byref(name)))
+    return name.value.decode()
 
 
 def profile_events(start=None, stop=None) -> None:

@@ -477,7 +477,46 @@ tq_status check_search(int64_t nq, int64_t n, int d, int bits, int k) {
   if (d > 2048) return fail(TQ_EUNSUPPORTED, "tq_search: d=%d > 2048 is not supported by this build", d);
   return TQ_OK;
 }
+
+// The scans tq_search dispatches to.
+enum class Scan { kStream, kRing, kFold, kMma, kTmExact, kTmFp16 };
+
+// The one a search of these sizes takes on the calling thread's path.
+tq_status pick_scan(int64_t nq, int64_t n, int d, int bits, int k, bool filtered, Scan* out) {
+  const int path = tq::search_path();
+  const bool can_mma = tq::mma_supported(bits, d, k);
+  if (path == TQ_PATH_MMA && !can_mma)
+    return fail(TQ_EUNSUPPORTED, "tq_search: the tensor-core scan needs bits 2/4/8, d %% 64 == 0 and k <= %d",
+                tq::kMaxKMma);
+  if (path == TQ_PATH_LUT_FOLD && !tq::fold_supported(bits, d, k, n))
+    return fail(TQ_EUNSUPPORTED,
+                "tq_search: the query-folded scan needs bits 4, d >= 256, k <= %d and n < 2^31 - 13312",
+                tq::kFoldMaxK);
+  *out = tq::scan_lut_is_ring(bits, d, k) ? Scan::kRing : Scan::kStream;
+  // (AUTO keeps the byte-pair scan from the folded one: on GB300 it is the faster
+  // of the two, 218 against 228 us per query at 999,000 x 1536)
+  if (path == TQ_PATH_LUT_FOLD) *out = Scan::kFold;
+  if (path == TQ_PATH_MMA) *out = Scan::kMma;
+  if (path != TQ_PATH_AUTO) return TQ_OK;
+  if (can_mma && nq >= tq::kMmaMinBatch)
+    *out = tq::scan_tm_supported(nq, n, d, bits, k, false, filtered) ? Scan::kTmFp16 : Scan::kMma;
+  else if (tq::scan_tm_supported(nq, n, d, bits, k, true, filtered))
+    *out = Scan::kTmExact;
+  return TQ_OK;
+}
 }  // namespace
+
+extern "C" tq_status tq_search_kernel(int64_t nq, int64_t n, int d, int bits, int k, int filtered, const char** name) {
+  if (!name) return fail(TQ_EINVAL, "tq_search_kernel: NULL name");
+  tq_status st = check_search(nq, n, d, bits, k);
+  Scan scan = Scan::kStream;
+  if (st == TQ_OK) st = pick_scan(nq, n, d, bits, k, filtered != 0, &scan);
+  if (st != TQ_OK) return st;
+  static const char* const names[] = {"k_scan_stream", "k_scan_ring", "k_scan_fold",
+                                      "k_scan_mma", "k_scan_tm (exact)", "k_scan_tm"};
+  *name = names[(int)scan];
+  return tq::ok();
+}
 
 extern "C" tq_status tq_search_workspace(int64_t nq, int64_t n, int d, int bits, int k,
                                          const tq_filter* filter, size_t* bytes) {
@@ -518,26 +557,9 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
     return fail(TQ_EINVAL, "tq_search_ex: a TQ+ calibration needs both mu and a");
   if (((uintptr_t)cal_mu & 3u) || ((uintptr_t)cal_a & 3u))
     return fail(TQ_EINVAL, "tq_search_ex: mu and a must be 4-byte aligned");
-  const int path = tq::search_path();
-  const bool can_mma = tq::mma_supported(bits, d, k);
-  if (path == TQ_PATH_MMA && !can_mma)
-    return fail(TQ_EUNSUPPORTED, "tq_search: the tensor-core scan needs bits 2/4/8, d %% 64 == 0 and k <= %d",
-                tq::kMaxKMma);
-  const bool use_mma = can_mma && (path == TQ_PATH_MMA || (path == TQ_PATH_AUTO && nq >= tq::kMmaMinBatch));
-  const bool can_fold = tq::fold_supported(bits, d, k, n);
-  if (path == TQ_PATH_LUT_FOLD && !can_fold)
-    return fail(TQ_EUNSUPPORTED,
-                "tq_search: the query-folded scan needs bits 4, d >= 256, k <= %d and n < 2^31 - 13312",
-                tq::kFoldMaxK);
-  // AUTO keeps the byte-pair scan: on GB300 it is the faster of the two (218
-  // against 228 us per query at 999,000 x 1536)
-  const bool use_fold = !use_mma && can_fold && path == TQ_PATH_LUT_FOLD;
-  // AUTO: the small-batch tensor-core scan, exact (bounds, then float32
-  // scores) for batches the lookup scan would take, fp16 above
-  const bool filtered = filter != nullptr;
-  const bool tm_bound = path == TQ_PATH_AUTO && !use_mma && tq::scan_tm_supported(nq, n, d, bits, k, true, filtered);
-  const bool use_tm =
-      tm_bound || (path == TQ_PATH_AUTO && use_mma && tq::scan_tm_supported(nq, n, d, bits, k, false, filtered));
+  Scan scan = Scan::kStream;
+  if ((st = pick_scan(nq, n, d, bits, k, filter != nullptr, &scan)) != TQ_OK) return st;
+  const bool tm_bound = scan == Scan::kTmExact;
   const tq::SearchPlan p = tq::plan_search(nq, n, d, bits, k, filter);
   if (ws_bytes < p.total)
     return fail(TQ_EINVAL, "tq_search: workspace of %zu bytes, %zu needed", ws_bytes, p.total);
@@ -558,7 +580,7 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
                                                   status, counters, p.n_cnt, s)
                            : tq::launch_rotate(Q, nq, d, R, qrot, status, counters, p.n_cnt, s);
   if (e == cudaSuccess && cal_mu) e = tq::launch_calib_query(qrot, nq, d, cal_mu, cal_a, bias, s);
-  if (use_tm) {
+  if (scan == Scan::kTmExact || scan == Scan::kTmFp16) {
     float* lows = reinterpret_cast<float*>(ws + p.off_lows);
     int* gate = reinterpret_cast<int*>(ws + p.off_gate);
     if (e == cudaSuccess && filter)
@@ -582,7 +604,7 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
     } else if (e == cudaSuccess) {
       e = tq::launch_merge(cs, ci, nq, p.grid_tm * k, k, ext_ids, out_ids, out_scores, s);
     }
-  } else if (use_mma) {
+  } else if (scan == Scan::kMma) {
     if (e == cudaSuccess && filter) e = tq::launch_allow_bits(filter->f, allow_off, allow_tenants, nq, allow, s);
     if (e == cudaSuccess)
       e = tq::launch_scan_mma(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
@@ -594,7 +616,7 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
     if (e == cudaSuccess) e = tq::launch_merge(cs, ci, nq, p.grid_mma * k, k, ext_ids, out_ids, out_scores, s);
   } else {
     if (e == cudaSuccess && filter) e = tq::launch_filter_prep(filter->f, allow_off, allow_tenants, nq, allow, bmask, s);
-    if (e == cudaSuccess && use_fold)
+    if (e == cudaSuccess && scan == Scan::kFold)
       e = tq::launch_scan_fold(qrot, nq, d, centroids, codes, scale, n, deleted, filter ? &filter->f : nullptr,
                                allow, bmask, k, p.grid_fold, cs, ci, status, counters, ext_ids, out_ids,
                                out_scores, bias, s, (cudaEvent_t)tq::profile_start(),
@@ -602,7 +624,7 @@ extern "C" tq_status tq_search_ex(const float* Q, int64_t nq, int d, const float
     else if (e == cudaSuccess)
       e = tq::launch_scan_lut(qrot, nq, d, centroids, bits, codes, scale, n, deleted,
                               filter ? &filter->f : nullptr, allow, bmask,
-                              path == TQ_PATH_LUT_FIXED && d >= tq::kFixMinD,
+                              tq::search_path() == TQ_PATH_LUT_FIXED && d >= tq::kFixMinD,
                               k, p.grid_lut, cs, ci, status, counters, ext_ids, out_ids, out_scores, bias,
                               nullptr, s, (cudaEvent_t)tq::profile_start(), (cudaEvent_t)tq::profile_stop());
   }

@@ -95,6 +95,7 @@ cudaError_t launch_filter_raw_ids(const FilterDev& f, uint32_t* raw, cudaStream_
 // per-query term, added to each raw score before the per-vector scale.  `gate`
 // [nq] (nullable; not for 3-bit codes): only queries with gate[q] != 0 are searched.
 int scan_lut_grid_x(int64_t nq, int64_t n, int k, int bits, int d);
+bool scan_lut_is_ring(int bits, int d, int k);  // fed by bulk copies (k_scan_ring), not k_scan_stream
 int64_t scan_lut_max_lists(int64_t nq, int64_t n, int k, int bits, int d);  // of any batch of up to nq queries
 cudaError_t launch_scan_lut(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
                             const uint8_t* codes, const float* scale, int64_t n, const uint32_t* del,

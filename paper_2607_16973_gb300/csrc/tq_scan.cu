@@ -1072,10 +1072,12 @@ cudaError_t scan_bits(int S, bool filt, bool fix, dim3 grid, size_t smem, cudaSt
 
 }  // namespace
 
+bool scan_lut_is_ring(int bits, int d, int k) { return ring_slots(bits, d, k) >= 2; }
+
 // One resident wave for a single query: one ring-scan CTA per SM, or two
 // register-fed CTAs.
 static int64_t lut_wave(int bits, int d, int k) {
-  return (int64_t)device_sm_count() * (ring_slots(bits, d, k) >= 2 ? 1 : 2);
+  return (int64_t)device_sm_count() * (scan_lut_is_ring(bits, d, k) ? 1 : 2);
 }
 
 // m * scan_lut_grid_x(m) for m <= nq is at most a wave and m - 1, and at most

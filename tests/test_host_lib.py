@@ -225,3 +225,43 @@ def test_encode_workspace_by_width(lib):
     sz = C.c_size_t()
     assert lib.tq_encode_workspace_for(1000, 1024, 5, C.byref(sz)) == _lib.TQ_EINVAL
     assert lib.tq_encode_workspace_for(1000, 1024, 4, None) == _lib.TQ_EINVAL
+
+
+@pytest.mark.parametrize("nq,n,d,bits,k,filtered,want", [
+    (1, 10_000, 1536, 4, 10, False, "k_scan_stream"),      # too little work for the exact small-batch search
+    (1, 100_000, 1536, 4, 10, False, "k_scan_tm (exact)"),
+    (1, 100_000, 1536, 4, 32, False, "k_scan_tm (exact)"),
+    (1, 50_000, 1536, 4, 32, False, "k_scan_stream"),
+    (1, 100_000, 1536, 4, 33, False, "k_scan_stream"),
+    (1, 100_000, 1536, 4, 10, True, "k_scan_stream"),
+    (15, 2048, 1536, 4, 10, False, "k_scan_tm (exact)"),
+    (15, 2047, 1536, 4, 10, False, "k_scan_stream"),
+    (16, 2048, 1536, 4, 10, False, "k_scan_tm"),
+    (32, 1, 256, 4, 32, True, "k_scan_tm"),
+    (33, 1, 256, 4, 32, True, "k_scan_mma"),
+    (16, 2048, 1600, 4, 10, False, "k_scan_mma"),
+    (16, 2048, 1536, 2, 64, False, "k_scan_mma"),
+    (16, 2048, 1536, 2, 65, False, "k_scan_stream"),
+    (1, 100_000, 1536, 3, 10, False, "k_scan_ring"),
+])
+def test_search_kernel(lib, nq, n, d, bits, k, filtered, want):
+    """The scan each size takes; the benchmark asks the same call."""
+    assert tq.search_kernel(nq, n, d, bits, k, filtered) == want
+
+
+def test_search_kernel_on_a_forced_path(lib):
+    try:
+        tq.set_search_path("mma")
+        assert tq.search_kernel(1, 100, 256, 4, 5) == "k_scan_mma"
+        with pytest.raises(tq.TQError):
+            tq.search_kernel(1, 100, 256, 4, 65)
+        tq.set_search_path("lut_fold")
+        assert tq.search_kernel(20, 100, 256, 4, 5) == "k_scan_fold"
+        with pytest.raises(tq.TQError):
+            tq.search_kernel(20, 100, 256, 2, 5)
+        tq.set_search_path("lut")
+        assert tq.search_kernel(20, 100_000, 1536, 4, 5) == "k_scan_stream"
+    finally:
+        tq.set_search_path("auto")
+    with pytest.raises(tq.TQError):
+        tq.search_kernel(1, 0, 256, 4, 5)
