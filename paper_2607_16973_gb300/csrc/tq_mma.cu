@@ -247,7 +247,15 @@ __device__ __forceinline__ uint4 decode8_4bit(uint32_t w, const uint32_t (&tl)[4
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-template <int BITS, int QT>
+constexpr int FEW_K = 8;  // from this k on the CTAs share list heads
+
+// FEW: a variant for k < FEW_K, whose lists are short: no list heads, no bisected
+// first threshold, no loads of many entries in flight, and so hardly a spilled
+// register in the epilogue (36 bytes of stores instead of 72 at 4 bits).  999,000 x
+// 1536, 4 bits, 128 queries: k = 1 477 -> 470 us, k = 5 494 -> 484; 300,001 x
+// 1024, 2 bits, 128 queries, k = 5 165 -> 148.  Not for 8-bit codes, whose decoders
+// set the pace and where it came out slower (64 queries, k = 1 815 -> 825 us).
+template <int BITS, int QT, bool FEW>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restrict__ qpack,
            const float* __restrict__ centroids, const float* __restrict__ scale,
@@ -542,7 +550,8 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
     // they are published: a CTA's best score or, for k > 32, its rank-th best
     const int rank = k <= 32 ? 1 : (k + 15) / 16, reach = (k + rank - 1) / rank;
     auto heads_turn = [&](int tile_i) {
-      return (tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= 8 && (int)gridDim.x >= reach;
+      return !FEW && (tile_i == 1 || tile_i == 4 || tile_i == 16 || tile_i == 64) && k >= FEW_K &&
+             (int)gridDim.x >= reach;
     };
     auto insert = [&](float sc, int v) {
       const uint64_t key = rank_key(sc, v);
@@ -552,7 +561,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       if (cnt < k) ++cnt;
       if (cnt < k) return;
       worst = ~0ull;
-#pragma unroll 8
+#pragma unroll(FEW ? 2 : 8)
       for (int i = 0; i < k; ++i) {
         const uint64_t o = i == slot ? key : lst[i * MMA_M];  // (not waiting for the store)
         wslot = o < worst ? i : wslot;
@@ -645,7 +654,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
               fn(c0, x);
             }
           };
-          if (k <= 16) {
+          if (FEW || k <= 16) {
             each([&](int c0, const float (&x)[16]) {
               if (q >= nq) return;
 #pragma unroll 1
@@ -792,7 +801,7 @@ k_scan_mma(const __grid_constant__ CUtensorMap codes_map, const __half* __restri
       // the merge takes its bounds; the others in any order
       uint64_t best = 0;
       int bi = 0;
-#pragma unroll 8
+#pragma unroll(FEW ? 2 : 8)
       for (int i = 0; i < cnt; ++i) {
         const uint64_t o = lst[i * MMA_M];
         bi = o > best ? i : bi;
@@ -851,11 +860,14 @@ cudaError_t launch_typed(const MmaPlan& P, const CUtensorMap& map, const __half*
     lists = nullptr;
   }
   const int gact = active_groups(P.ng, sub, P.cst);
-  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_scan_mma<BITS, QT>), (int)smem);
+  auto kernel = k_scan_mma<BITS, QT, false>;
+  if constexpr (BITS != 8)
+    if (k < FEW_K) kernel = k_scan_mma<BITS, QT, true>;
+  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)smem);
   if (e != cudaSuccess) return e;
   const int nqt = (nq + MMA_M - 1) / MMA_M;
   const dim3 grid((unsigned)grid_x, (unsigned)((nqt + QT - 1) / QT));
-  return launch_maybe_pdl(pdl, k_scan_mma<BITS, QT>, grid, dim3(NTHREADS), (size_t)smem, s, map, qpack, centroids,
+  return launch_maybe_pdl(pdl, kernel, grid, dim3(NTHREADS), (size_t)smem, s, map, qpack, centroids,
                           scale, del, dense, allow, words, bias, n, nq, d, k, P.cst, P.ast, P.rr, sub, P.ng, gact, cs,
                           ci, err, gth, heads, lists);
 }

@@ -25,6 +25,9 @@ def tdev(cuda_lib):
     (90_001, 40, 20, 4, 0.3),      # three tiles per CTA: heads read at the second; deleted rows
     (90_001, 130, 8, 2, 0.0),      # two query tiles, the smallest k that reads heads
     (60_000, 300, 33, 4, 0.999),   # fewer live rows per CTA than k; heads of rank 3
+    (90_001, 40, 7, 4, 0.3),       # the largest k of the kernel for short lists
+    (90_001, 130, 1, 3, 0.0),      # its smallest, two query tiles
+    (90_001, 40, 7, 8, 0.3),       # 8-bit codes have none: short lists in the general one
 ])
 def test_mma_lists(cuda_lib, tdev, n, nq, k, bits, dead):
     torch, T = tdev
@@ -35,7 +38,8 @@ def test_mma_lists(cuda_lib, tdev, n, nq, k, bits, dead):
     packed[n // 2: n // 2 + 40] = packed[0]      # ties, in rank order of the rows
     scale[n // 2: n // 2 + 40] = scale[0]
     R = O.rotation(d, 5).astype(np.float32)
-    c32 = O.codebook(d, bits, "beta").centroids32
+    # (the oracle's own 8-bit codebook takes minutes)
+    c32 = O.codebook(d, bits, "beta").centroids32 if bits < 8 else tq.codebook(d, bits)[0]
     Q = synth.gaussian_rows(nq, d, seed=nq)
     Q /= np.linalg.norm(Q, axis=1, keepdims=True)
     m, gone = None, np.zeros(n, bool)
