@@ -731,6 +731,20 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
 // (k_scan_stream's operations in its order) and the k best of those are the
 // result, unless a full list's last U reaches the k-th best score: a vector
 // that list dropped might belong to the result, so the gate opens.
+//
+// The keys sorted at the end hold, below ~id (whose top bit is always set and
+// left out), whether the score is -0: zeros of either sign rank by id, as in the
+// lookup scan, and come out as they were.
+__device__ __forceinline__ uint64_t result_key(float s, int id) {
+  return (rank_key(s, 0) & 0xFFFFFFFF00000000u) | ((uint32_t)~id << 1) |
+         (__float_as_uint(s) == 0x80000000u ? 1u : 0u);
+}
+__device__ __forceinline__ float result_score(uint64_t key) {
+  const float s = key_score(key);
+  return s == 0.f && (key & 1u) ? -0.f : s;
+}
+__device__ __forceinline__ int result_id(uint64_t key) { return (int)~(((uint32_t)key >> 1) | 0x80000000u); }
+
 constexpr int RS_NT = 1024;
 constexpr int RS_CAP = 1024;  // candidates one block scores
 constexpr int RS_PER = 5;     // list entries per thread: 152 lists of 32
@@ -833,11 +847,11 @@ k_rescore(const float* __restrict__ qrot, int d, const float* __restrict__ centr
     float tot = acc.x + acc.y;
 #pragma unroll
     for (int o = 16; o; o >>= 1) tot += __shfl_xor_sync(FULL, tot, o);
-    if (lane == 0) key[p] = rank_key((tot + bq) * sc, v);
+    if (lane == 0) key[p] = result_key((tot + bq) * sc, v);
   }
   int P = 32;
   while (P < ns) P <<= 1;
-  const uint64_t none = rank_key(-INFINITY, INT_MAX);
+  const uint64_t none = result_key(-INFINITY, INT_MAX);
   for (int i = ns + tid; i < P; i += RS_NT) key[i] = none;
   __syncthreads();
   if (P == 32) {
@@ -860,10 +874,10 @@ k_rescore(const float* __restrict__ qrot, int d, const float* __restrict__ centr
   }
   __syncthreads();
   if (tid < k) {
-    const int v = key_id(key[tid]);
+    const int v = result_id(key[tid]);
     const bool empty = v == INT_MAX;
     out_ids[(size_t)q * k + tid] = empty ? -1 : ext ? (int64_t)__ldg(ext + v) : (int64_t)v;
-    out_scores[(size_t)q * k + tid] = empty ? -INFINITY : key_score(key[tid]);
+    out_scores[(size_t)q * k + tid] = empty ? -INFINITY : result_score(key[tid]);
   }
   const float kth = key_score(key[k - 1]);
   // each thread still holds the lists' last entries it loaded

@@ -121,6 +121,26 @@ def test_exact_search_on_odd_values(cuda_lib, tdev, change):
     assert np.array_equal(ids, ids_l) and np.array_equal(sc, sc_l, equal_nan=True)
 
 
+def test_exact_search_keeps_the_sign_of_zero(cuda_lib, tdev):
+    """Rows of scale 0 score 0 or -0, by the sign of their product, and rank by
+    id among them: the best results here, all other scores being negative."""
+    torch, T = tdev
+    tq = cuda_lib
+    d, n, k = 512, 40_000, 8
+    packed, scale, R, Q = _data(n, d, 1, seed=61)
+    c32, _ = _cb(d)
+    dot = c32.astype(np.float64)[O.unpack(packed, d, 4)] @ (R.astype(np.float64) @ Q[0])
+    scale = (-np.abs(scale) * np.sign(dot)).astype(np.float32)
+    zero = np.concatenate([np.nonzero(dot > 0)[0][100:500:100], np.nonzero(dot < 0)[0][100:400:100]])
+    scale[zero] = 0.0
+    a = (T(Q), T(R), T(c32), 4, T(packed), T(scale), k)
+    assert tq.search_kernel(1, n, d, 4, k) == "k_scan_tm (exact)"
+    ids, sc = _search(tq, torch, "auto", *a)
+    ids_l, sc_l = _search(tq, torch, "lut", *a)
+    assert np.array_equal(ids[0, :7], np.sort(zero)) and np.signbit(sc_l[0, :7]).sum() == 3
+    assert np.array_equal(ids, ids_l) and np.array_equal(sc.view(np.int32), sc_l.view(np.int32))
+
+
 def test_exact_search_with_deleted_rows_and_calibration(cuda_lib, tdev):
     torch, T = tdev
     tq = cuda_lib
