@@ -43,9 +43,11 @@ int& fail_allocs();
 
 inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
 inline int64_t row_bytes(int d, int bits) { return (int64_t)d * bits / 8; }
-// Tiles of `rows` rows that n rows take, without forming a number above n (n
-// goes up to 2^31 - 2 in int arithmetic; n + rows - 1 would wrap there).
-constexpr int row_tiles(int n, int rows) { return n / rows + (n % rows != 0 ? 1 : 0); }
+// Tiles of `rows` rows that n rows take (n goes up to 2^31 - 2, where n + rows - 1
+// would wrap as an int).
+constexpr int row_tiles(int n, int rows) {
+  return (int)(((unsigned)n + (unsigned)rows - 1u) / (unsigned)rows);
+}
 static_assert(row_tiles(0x7FFFFFFE, 128) == 1 << 24 && row_tiles(0x7FFFFFFE, 4) == 1 << 29 &&
                   row_tiles(128, 128) == 1 && row_tiles(129, 128) == 2,
               "row tiles");
