@@ -90,6 +90,37 @@ def test_encode_h_values_out_of_range(cuda_lib, tdev):
     assert np.mean(codes.cpu().numpy()[20:] != codes_t[20:]) < 2e-4
 
 
+@pytest.mark.parametrize("bits", [2, 4, 8])
+@pytest.mark.parametrize("how", ["close", "equal", "infinite"])
+def test_encode_h_boundaries_no_cell_separates(cuda_lib, tdev, bits, how):
+    """Two boundaries in one lookup cell (close or equal), or a range that is not
+    finite: the codes come from the search, as the TF32 encoder's do."""
+    torch, dev, T = tdev
+    tq = cuda_lib
+    n, d = 120, 1024
+    X, R = synth.gaussian_rows(n, d, seed=5), O.rotation(d, 7).astype(np.float32)
+    c32, t32 = (a.copy() for a in tq.codebook(d, bits)[:2])
+    m = len(t32) // 2
+    if how == "infinite":
+        t32[0], t32[-1] = -np.inf, np.inf
+    else:
+        t32[m] = t32[m - 1] + (np.float32(1e-6) if how == "close" else 0)
+    plan = tq.encode_plan(T(R))
+    codes, scale = tq.encode(T(X), None, T(c32), T(t32), bits, "norm", plan=plan)
+    codes, scale = codes.cpu().numpy(), scale.cpu().numpy()
+    codes_t, scale_t = _tf32(tq, torch, T(X), plan, T(c32), T(t32), bits, "norm")
+    a, b = (O.unpack(x, d, bits).astype(np.int64) for x in (codes, codes_t))
+    # where they differ the coordinate lies next to a boundary: a cell away, or two across the narrow one
+    assert np.abs(a - b).max() <= (2 if how != "infinite" else 1) and np.mean(a != b) < (1e-3 if bits == 8 else 2e-4)
+    same = (a == b).all(axis=1)
+    assert same.any() and np.allclose(scale[same], scale_t[same], rtol=2e-6)
+    y = (X.astype(np.float64) / np.linalg.norm(X, axis=1, keepdims=True)) @ R.T.astype(np.float64)
+    want = np.searchsorted(t32.astype(np.float64), y)  # boundaries below y
+    off = a != want
+    near = np.abs(y[..., None] - t32[None, None].astype(np.float64)).min(axis=-1) < 1e-5
+    assert np.all(near[off])
+
+
 def test_encode_h_workspace(cuda_lib, tdev):
     """A kept workspace is reused, one that is too small is refused."""
     torch, dev, T = tdev

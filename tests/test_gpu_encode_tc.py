@@ -3,7 +3,10 @@ in TF32 with a three-product split) against the oracle's float64 encode, with
 the same checks as the FFMA encoder: codes equal except one-cell flips within
 the boundary window, scalars to the tolerance of each scale mode.  The sizes
 reach several panels per CTA (more panels than SMs), partial last chunks of
-256 coordinates, panels with a ragged tail and rows of zeros.
+256 coordinates, panels with a ragged tail and rows of zeros.  Every case runs
+both without a workspace, which is this encoder at every d, and as encode()
+runs it by default: from d = 1024 on (8-bit codes 768) the fp16 encoder, which
+has the same bounds.
 
 Its y carries about 1e-7 of error at d = 1536 (at most ~1e-6), mostly from
 the float32 accumulation inside the tensor cores, against ~5e-9 for the FFMA
@@ -46,10 +49,13 @@ def _rate(bits):
     return 1e-3 if bits == 8 else 1e-4
 
 
-def _planned(tq, T, X, R, c32, t32, bits, mode="norm", calib=None):
+both = pytest.mark.parametrize("workspace", [False, None], ids=["tf32", "default"])
+
+
+def _planned(tq, T, X, R, c32, t32, bits, mode="norm", calib=None, workspace=False):
     import torch
     plan = tq.encode_plan(T(R))
-    codes, scale = tq.encode(T(X), None, T(c32), T(t32), bits, mode, plan=plan, calib=calib)
+    codes, scale = tq.encode(T(X), None, T(c32), T(t32), bits, mode, plan=plan, calib=calib, workspace=workspace)
     tq.encode_check(plan)
     torch.cuda.synchronize()
     return codes.cpu().numpy(), scale.cpu().numpy()
@@ -75,9 +81,10 @@ def test_plan_is_a_tf32_split(cuda_lib, tdev):
     assert np.all(np.abs(hi.astype(np.float64) + lo - r) <= 2.0 ** -22 * np.abs(r))
 
 
+@both
 @pytest.mark.parametrize("bits", [2, 3, 4, 8])
 @pytest.mark.parametrize("mode", ["norm", "none", "unbiased"])
-def test_encode_planned_parity(cuda_lib, tdev, bits, mode):
+def test_encode_planned_parity(cuda_lib, tdev, bits, mode, workspace):
     torch, dev, T = tdev
     tq = cuda_lib
     d, n = 1536, 2077                       # 16 panels of 128 rows + a ragged 29
@@ -87,13 +94,14 @@ def test_encode_planned_parity(cuda_lib, tdev, bits, mode):
     R = O.rotation(d, 1536).astype(np.float32)
     c32, t32 = _cb(d, bits)
     enc = O.encode(X, R, c32, t32, bits, mode)
-    codes, scale = _planned(tq, T, X, R, c32, t32, bits, mode)
+    codes, scale = _planned(tq, T, X, R, c32, t32, bits, mode, workspace=workspace)
     check_encode(codes, scale, X, enc, c32, t32, d, bits, mode, max_rate=_rate(bits))
     assert np.all(codes[5] == enc.packed[5]) and scale[5] == 0.0
 
 
+@both
 @pytest.mark.parametrize("bits,mode", [(4, "norm"), (3, "unbiased")])
-def test_encode_planned_many_panels(cuda_lib, tdev, bits, mode):
+def test_encode_planned_many_panels(cuda_lib, tdev, bits, mode, workspace):
     """More panels than SMs: each CTA runs 2-3 panels, so the per-panel norm
     and sum buffers and both accumulator sets are reused."""
     torch, dev, T = tdev
@@ -104,12 +112,13 @@ def test_encode_planned_many_panels(cuda_lib, tdev, bits, mode):
     R = O.rotation(d, 1536).astype(np.float32)
     c32, t32 = _cb(d, bits)
     enc = O.encode(X, R, c32, t32, bits, mode)
-    codes, scale = _planned(tq, T, X, R, c32, t32, bits, mode)
+    codes, scale = _planned(tq, T, X, R, c32, t32, bits, mode, workspace=workspace)
     check_encode(codes, scale, X, enc, c32, t32, d, bits, mode)
 
 
+@both
 @pytest.mark.parametrize("d", [128, 160, 384, 2048, 4096])
-def test_encode_planned_dims(cuda_lib, tdev, d):
+def test_encode_planned_dims(cuda_lib, tdev, d, workspace):
     """One partial chunk (128, 160), a partial last chunk (384), several full
     chunks (2048, 4096)."""
     torch, dev, T = tdev
@@ -119,12 +128,13 @@ def test_encode_planned_dims(cuda_lib, tdev, d):
     R = O.rotation(d, 11).astype(np.float32)
     c32, t32 = _cb(d, bits)
     enc = O.encode(X, R, c32, t32, bits)
-    codes, scale = _planned(tq, T, X, R, c32, t32, bits)
+    codes, scale = _planned(tq, T, X, R, c32, t32, bits, workspace=workspace)
     check_encode(codes, scale, X, enc, c32, t32, d, bits, "norm")
 
 
+@both
 @pytest.mark.parametrize("n", [1, 5, 127, 128, 129])
-def test_encode_planned_small_batches(cuda_lib, tdev, n):
+def test_encode_planned_small_batches(cuda_lib, tdev, n, workspace):
     """Fewer rows than one panel (the X tile is zero-filled past row n) and
     the panel edge."""
     torch, dev, T = tdev
@@ -134,11 +144,12 @@ def test_encode_planned_small_batches(cuda_lib, tdev, n):
     R = O.rotation(d, 1536).astype(np.float32)
     c32, t32 = _cb(d, bits)
     enc = O.encode(X, R, c32, t32, bits)
-    codes, scale = _planned(tq, T, X, R, c32, t32, bits)
+    codes, scale = _planned(tq, T, X, R, c32, t32, bits, workspace=workspace)
     check_encode(codes, scale, X, enc, c32, t32, d, bits, "norm")
 
 
-def test_encode_planned_empty_and_offsets(cuda_lib, tdev):
+@both
+def test_encode_planned_empty_and_offsets(cuda_lib, tdev, workspace):
     """n = 0 is a no-op; codes and scale written into a larger array at a row
     offset land only in their rows."""
     torch, dev, T = tdev
@@ -148,12 +159,13 @@ def test_encode_planned_empty_and_offsets(cuda_lib, tdev):
     c32, t32 = _cb(d, bits)
     plan = tq.encode_plan(T(R))
     empty = torch.empty((0, d), dtype=torch.float32, device=dev)
-    codes, scale = tq.encode(empty, None, T(c32), T(t32), bits, plan=plan)
+    codes, scale = tq.encode(empty, None, T(c32), T(t32), bits, plan=plan, workspace=workspace)
     assert codes.shape == (0, d * bits // 8)
     X = synth.mixture_corpus(n, d, 4, seed=3)
     big_c = torch.full((n + 64, d * bits // 8), 0xAB, dtype=torch.uint8, device=dev)
     big_s = torch.full((n + 64,), -7.0, dtype=torch.float32, device=dev)
-    tq.encode(T(X), None, T(c32), T(t32), bits, "norm", big_c[32:32 + n], big_s[32:32 + n], plan=plan)
+    tq.encode(T(X), None, T(c32), T(t32), bits, "norm", big_c[32:32 + n], big_s[32:32 + n], plan=plan,
+              workspace=workspace)
     torch.cuda.synchronize()
     bc, bs = big_c.cpu().numpy(), big_s.cpu().numpy()
     assert np.all(bc[:32] == 0xAB) and np.all(bc[32 + n:] == 0xAB)
@@ -162,8 +174,9 @@ def test_encode_planned_empty_and_offsets(cuda_lib, tdev):
     check_encode(bc[32:32 + n], bs[32:32 + n], X, enc, c32, t32, d, bits, "norm")
 
 
+@both
 @pytest.mark.parametrize("bits", [3, 4])
-def test_encode_planned_tqplus(cuda_lib, tdev, bits):
+def test_encode_planned_tqplus(cuda_lib, tdev, bits, workspace):
     """A TQ+ calibration (the oracle's, rounded to float32, on both sides)."""
     torch, dev, T = tdev
     tq = cuda_lib
@@ -177,11 +190,12 @@ def test_encode_planned_tqplus(cuda_lib, tdev, bits):
     cal = O.calibration32(O.calibrate(X[:500], R))
     enc = O.encode(X, R, c32, t32, bits, "unbiased", calib=cal)
     codes, scale = _planned(tq, T, X, R, c32, t32, bits, "unbiased",
-                            calib=(T(cal.mu.astype(np.float32)), T(cal.a.astype(np.float32))))
+                            calib=(T(cal.mu.astype(np.float32)), T(cal.a.astype(np.float32))), workspace=workspace)
     check_encode(codes, scale, X, enc, c32, t32, d, bits, "unbiased", calib=cal)
 
 
-def test_encode_planned_matches_ffma_encoder(cuda_lib, tdev):
+@both
+def test_encode_planned_matches_ffma_encoder(cuda_lib, tdev, workspace):
     """The two encoders differ only in the rounding of y: their codes agree
     except for one-cell flips, at most a few in 10^5."""
     torch, dev, T = tdev
@@ -191,7 +205,7 @@ def test_encode_planned_matches_ffma_encoder(cuda_lib, tdev):
     R = O.rotation(d, 1536).astype(np.float32)
     c32, t32 = _cb(d, bits)
     a, sa = tq.encode(T(X), T(R), T(c32), T(t32), bits)
-    b, sb = _planned(tq, T, X, R, c32, t32, bits)
+    b, sb = _planned(tq, T, X, R, c32, t32, bits, workspace=workspace)
     ua = O.unpack(a.cpu().numpy(), d, bits).astype(np.int64)
     ub = O.unpack(b, d, bits).astype(np.int64)
     diff = ua != ub
@@ -199,3 +213,23 @@ def test_encode_planned_matches_ffma_encoder(cuda_lib, tdev):
     assert diff.mean() < 1e-4
     same = ~diff.any(axis=1)
     assert np.allclose(sa.cpu().numpy()[same], sb[same], rtol=2e-6)
+
+
+@pytest.mark.parametrize("d,bits,tqplus", [(384, 2, False), (384, 3, True), (384, 4, True), (768, 4, False),
+                                           (768, 2, True), (640, 8, True)])
+def test_encode_planned_where_it_is_the_default(cuda_lib, tdev, d, bits, tqplus):
+    """Below d = 1024 (8-bit codes 768) encode() takes this encoder: every width,
+    with and without a TQ+ calibration, with more panels than SMs."""
+    torch, dev, T = tdev
+    tq = cuda_lib
+    n, mode = 153 * 128 + 5, "unbiased" if tqplus else "norm"
+    assert tq.encode_workspace(n, d, bits) == 0
+    X = synth.mixture_corpus(n, d, 16, seed=d + bits)
+    X[n - 1] = 0.0
+    R = O.rotation(d, 7).astype(np.float32)
+    c32, t32 = _cb(d, bits) if bits < 8 else tq.codebook(d, bits)[:2]  # (the oracle's own 8-bit one takes minutes)
+    cal = O.calibration32(O.calibrate(X[:500], R)) if tqplus else None
+    enc = O.encode(X, R, c32, t32, bits, mode, calib=cal)
+    calib = (T(cal.mu.astype(np.float32)), T(cal.a.astype(np.float32))) if tqplus else None
+    codes, scale = _planned(tq, T, X, R, c32, t32, bits, mode, calib, workspace=None)
+    check_encode(codes, scale, X, enc, c32, t32, d, bits, mode, max_rate=_rate(bits), calib=cal)

@@ -601,3 +601,28 @@ def test_filter_every_tenant_equals_unfiltered_mma(cuda_lib, torch_dev, filtered
     finally:
         filt.close()
     assert np.array_equal(ids_f, ids_u) and np.array_equal(sc_f, sc_u)
+
+
+def test_filter_bitmap_beyond_shared_memory(cuda_lib, torch_dev):
+    """More than 393,216 tenants: a query's allow bitmap is more than 48 KB, so
+    the bitmaps and block masks are written by two kernels instead of one."""
+    torch, dev = torch_dev
+    tq = cuda_lib
+    n, d, bits, nq, k = 393_300, 32, 2, 3, 10
+    tenants = (np.random.default_rng(5).permutation(n).astype(np.uint32) + 11) * np.uint32(7)
+    packed, scale = synth.random_codes(n, d * bits // 8, seed=1), synth.random_scales(n, seed=1)
+    R = O.rotation(d, 3).astype(np.float32)
+    c32, _ = _cb(d, bits)
+    Q = synth.gaussian_rows(nq, d, seed=1)
+    lists = [tenants[5:25], tenants[n - 100:], np.append(tenants[:4], [3, 4]).astype(np.uint32)]
+    off = np.cumsum([0] + [len(v) for v in lists]).astype(np.int64)
+    ten = np.concatenate(lists)
+    filt = tq.Filter(_t(torch, dev, tenants.view(np.int32)), block=64)
+    ids, sc = tq.search(_t(torch, dev, Q), _t(torch, dev, R), _t(torch, dev, c32), bits, _t(torch, dev, packed),
+                        _t(torch, dev, scale), k, filter=filt, allow_off=_t(torch, dev, off),
+                        allow_tenants=_t(torch, dev, ten.view(np.int32)))
+    torch.cuda.synchronize()
+    ref = O.search(Q, R, c32, bits, packed, scale, k, d, tenant_ids=tenants, allow_off=off, allow_ids=ten)
+    allowed = np.stack([np.isin(tenants, v) for v in lists])
+    check_topk(ids.cpu().numpy(), sc.cpu().numpy(), ref.ids, ref.scores64, allowed, k, TOL_LUT)
+    filt.close()

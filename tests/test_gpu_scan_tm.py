@@ -243,3 +243,57 @@ def test_profile_events_cover_the_whole_exact_scan(cuda_lib, tdev):
             times.append(ev[0].elapsed_time(ev[1]))
         ms[path] = sorted(times)[3]
     assert ms["auto"] > 1.3 * ms["lut"], ms
+
+
+def test_exact_search_filtered_without_a_tile(cuda_lib, tdev):
+    """Allowlists that name no tenant of the corpus: no CTA has a tile to scan."""
+    torch, T = tdev
+    tq = cuda_lib
+    d, n, nq, k = 512, 60_001, 6, 10
+    packed, scale, R, Q = _data(n, d, nq, seed=43)
+    tenants, values = synth.zipf_tenants(n, 100)
+    flt = tq.Filter(T(tenants.view(np.int32)), block=64)
+    assert tq.search_kernel(nq, n, d, 4, k, filtered=True) == "k_scan_tm (exact)"
+    none = np.setdiff1d(np.arange(200, dtype=np.uint32), values)[:40]
+    for lists in ([none[:0]] * nq, [none[:2], none[:0], none[2:3], none, none[5:9], none[:1]]):
+        off = np.cumsum([0] + [len(v) for v in lists]).astype(np.int64)
+        ten = np.append(np.concatenate(lists), 1).astype(np.uint32)  # (never an empty tensor)
+        ids, sc = _search(tq, torch, "auto", T(Q), T(R), T(_cb(d)[0]), 4, T(packed), T(scale), k, filter=flt,
+                          allow_off=T(off), allow_tenants=T(ten.view(np.int32)))
+        assert np.all(ids == -1) and np.all(np.isneginf(sc))
+
+
+@pytest.mark.parametrize("d", [256, 2048])
+@pytest.mark.parametrize("nq", [16, 32])
+def test_accumulation_error_the_bounds_allow(cuda_lib, tdev, d, nq):
+    """The exact search's bound gives the MMAs' float32 accumulation an error of
+    d * 2^-23 of sum |q c|.  Here every operand is an fp16 number, so the fp16
+    search's scores are off by that error alone: products far apart in
+    magnitude, whose small ones are cut when aligned to the large."""
+    torch, T = tdev
+    tq = cuda_lib
+    rng = np.random.default_rng(d)
+    mag = np.array([2.0 ** -13, 2.0 ** -12, 1.5 * 2.0 ** -12, 2.0 ** -9, 2.0 ** -5, 0.25, 1.0, 1.9990234375])
+    c = np.sort(np.concatenate([-mag, mag])).astype(np.float32)
+    n = 32
+    codes = rng.integers(0, 16, (n, d))
+    small, one = 9, 14                       # codes of 2^-12 and 1
+    codes[:8] = small
+    codes[0, 0] = codes[1, d - 1] = codes[2, d // 2] = codes[3, ::16] = codes[4, 15::16] = one
+    codes[5, ::2] = 15 - small               # -2^-12 between them: the cut sums have opposite signs
+    codes[5, 1] = one
+    Q = np.where(rng.random((nq, d)) < 0.5, rng.choice(mag, (nq, d)), rng.uniform(-1, 1, (nq, d)).astype(np.float16))
+    Q[:4] = 2.0 ** -12
+    Q[0, 0] = Q[1, d - 1] = Q[2, d // 2] = 1.0
+    Q[3, ::16] = 1.0
+    Q[4], Q[5] = 1.0, np.where(np.arange(d) % 3 == 0, -1.0, 1.0)
+    Q = Q.astype(np.float32)
+    assert np.array_equal(Q, Q.astype(np.float16)) and np.array_equal(c, c.astype(np.float16))
+    assert tq.search_kernel(nq, n, d, 4, n) == "k_scan_tm"
+    ids, sc = _search(tq, torch, "auto", T(Q), T(np.eye(d, dtype=np.float32)), T(c), 4,
+                      T(O.pack(codes.astype(np.uint8), 4)), None, n)
+    rec = c.astype(np.float64)[codes]
+    exact = np.take_along_axis(Q.astype(np.float64) @ rec.T, ids, axis=1)
+    total = np.take_along_axis(np.abs(Q.astype(np.float64)) @ np.abs(rec).T, ids, axis=1)
+    share = np.abs(sc - exact) / (d * 2.0 ** -23 * total)
+    assert share.max() <= 1.0, share.max()
