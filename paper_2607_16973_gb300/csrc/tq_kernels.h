@@ -142,7 +142,7 @@ cudaError_t launch_merge_global(const float* cand_s, const int64_t* cand_i, int6
 bool mma_supported(int bits, int d, int k);
 int scan_mma_grid_x(int64_t nq, int64_t n, int k, int bits);
 size_t mma_qpack_bytes(int64_t nq, int d);
-size_t mma_list_bytes(int64_t nq, int bits, int k, int grid_x);  // the `lists` scratch: a list per query and CTA
+size_t mma_list_bytes(int64_t nq, int bits, int k, int grid_x);  // the `lists` scratch: a list per query and CTA, where they do not fit in shared memory
 cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
                             const uint8_t* codes, const float* scale, int64_t n, const uint32_t* del,
                             const uint32_t* dense, const uint32_t* allow_bits, int words, const float* bias,

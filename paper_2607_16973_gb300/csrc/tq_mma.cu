@@ -187,29 +187,24 @@ constexpr int MIN_PREFETCH_KB = 6;  // K-blocks of codes in flight (HBM latency)
 template <int BITS>
 MmaPlan mma_plan(int64_t nq) {
   MmaPlan best;
-  // first pass as above; the second relaxes the prefetch floor and allows
-  // fewer groups (large k at 8 bits needs the room for its lists)
-  for (int pass = 0; pass < 2; ++pass) {
-    const int min_pf = pass == 0 ? MIN_PREFETCH_KB : 2;
-    for (int qt = (nq > MMA_M ? 2 : 1); qt >= 1; --qt) {
-      const int gmax = qt == 2 ? dec_groups<2>() : dec_groups<1>();
-      for (int ng = gmax; ng >= 2; --ng) {
-        for (int rr = RAW_ROW_MAX; rr >= 64; rr >>= 1) {
-          const int sub = tile_sub(BITS, rr);  // for d a multiple of 256
-          for (int ast = 3; ast >= 2; --ast) {
-            for (int cst = MAX_CST; cst >= 2; --cst) {
-              if (cst * sub < min_pf || active_groups(ng, sub, cst) != ng) continue;
-              const uint32_t need = qt == 2 ? mma_smem_layout<BITS, 2>(cst, ast, rr, ng).total
-                                            : mma_smem_layout<BITS, 1>(cst, ast, rr, ng).total;
-              if (need <= kMaxDynSmem) {
-                best.qt = qt;
-                best.cst = cst;
-                best.ast = ast;
-                best.rr = rr;
-                best.ng = ng;
-                best.smem = need;
-                return best;
-              }
+  for (int qt = (nq > MMA_M ? 2 : 1); qt >= 1; --qt) {
+    const int gmax = qt == 2 ? dec_groups<2>() : dec_groups<1>();
+    for (int ng = gmax; ng >= 2; --ng) {
+      for (int rr = RAW_ROW_MAX; rr >= 64; rr >>= 1) {
+        const int sub = tile_sub(BITS, rr);  // for d a multiple of 256
+        for (int ast = 3; ast >= 2; --ast) {
+          for (int cst = MAX_CST; cst >= 2; --cst) {
+            if (cst * sub < MIN_PREFETCH_KB || active_groups(ng, sub, cst) != ng) continue;
+            const uint32_t need = qt == 2 ? mma_smem_layout<BITS, 2>(cst, ast, rr, ng).total
+                                          : mma_smem_layout<BITS, 1>(cst, ast, rr, ng).total;
+            if (need <= kMaxDynSmem) {
+              best.qt = qt;
+              best.cst = cst;
+              best.ast = ast;
+              best.rr = rr;
+              best.ng = ng;
+              best.smem = need;
+              return best;
             }
           }
         }
@@ -219,6 +214,11 @@ MmaPlan mma_plan(int64_t nq) {
   best.smem = 0;  // does not fit
   return best;
 }
+
+// Bytes of the CTA's lists: they go behind the rest in shared memory where they
+// fit, else to global memory.
+uint32_t list_bytes(const MmaPlan& P, int k) { return (uint32_t)P.qt * k * MMA_M * sizeof(uint64_t); }
+bool lists_in_smem(const MmaPlan& P, int k) { return P.smem + list_bytes(P, k) <= kMaxDynSmem; }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;
@@ -854,9 +854,8 @@ cudaError_t launch_typed(const MmaPlan& P, const CUtensorMap& map, const __half*
                          int words, const float* bias, int n, int nq, int d, int k, int sub, int grid_x, float* cs,
                          int* ci, int* err, uint32_t* gth, uint32_t* heads, uint64_t* lists, bool pdl, cudaStream_t s) {
   uint32_t smem = P.smem;
-  const uint32_t room = (uint32_t)QT * k * MMA_M * sizeof(uint64_t);
-  if (smem + room <= kMaxDynSmem) {
-    smem += room;
+  if (lists_in_smem(P, k)) {
+    smem += list_bytes(P, k);
     lists = nullptr;
   }
   const int gact = active_groups(P.ng, sub, P.cst);
@@ -901,9 +900,10 @@ size_t mma_qpack_bytes(int64_t nq, int d) {
 }
 
 size_t mma_list_bytes(int64_t nq, int bits, int k, int grid_x) {
-  const int qt = plan_for(bits, nq).qt;
-  const int64_t groups = ((nq + MMA_M - 1) / MMA_M + qt - 1) / qt;
-  return (size_t)groups * grid_x * qt * k * MMA_M * sizeof(uint64_t);
+  const MmaPlan P = plan_for(bits, nq);
+  if (lists_in_smem(P, k)) return 0;
+  const int64_t groups = ((nq + MMA_M - 1) / MMA_M + P.qt - 1) / P.qt;
+  return (size_t)groups * grid_x * list_bytes(P, k);
 }
 
 cudaError_t launch_scan_mma(const float* qrot, int64_t nq, int d, const float* centroids, int bits,
