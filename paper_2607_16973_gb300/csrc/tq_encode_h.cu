@@ -99,15 +99,6 @@ HWs h_ws(int64_t n, int d) {
   return w;
 }
 
-__device__ __forceinline__ float h_pow2(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-__device__ __forceinline__ int h_exp(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFFu) - 127; }
-
-__device__ __forceinline__ void h_mma(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc));
-}
 __device__ __forceinline__ void h_st16(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
@@ -116,12 +107,6 @@ __device__ __forceinline__ void h_st16(uint32_t taddr, const uint32_t (&r)[16]) 
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
-__device__ __forceinline__ bool h_elect() {
-  uint32_t p;
-  asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n selp.u32 %0, 1, 0, e;\n}" : "=r"(p));
-  return p != 0;
-}
-
 // Before the encode: blocks 0 .. d-1 scale and convert a row of the plan's
 // R_hi and R_lo (TF32 values, so the conversions are exact up to the low
 // range); the others take a row of X per warp: its norm (step 1; float
@@ -147,7 +132,7 @@ k_encode_prep(const float* __restrict__ X, int64_t n, int d, const unsigned char
     __syncthreads();
     for (int w = 0; w < 8; ++w) mx = fmaxf(mx, red[w]);
     // (a row of zeros, or one out of float32's middle range, is converted as it is)
-    const float s = mx >= 0x1p-100f && mx <= 0x1p100f ? h_pow2(13 - h_exp(mx)) : 1.0f;
+    const float s = mx >= 0x1p-100f && mx <= 0x1p100f ? pow2f(13 - exp2_of(mx)) : 1.0f;
     if (tid == 0) rinv[blockIdx.x] = 1.0f / s;
     uint2* oh = reinterpret_cast<uint2*>(r16 + (size_t)blockIdx.x * d);
     uint2* ol = reinterpret_cast<uint2*>(r16 + ((size_t)d + blockIdx.x) * d);
@@ -187,7 +172,7 @@ k_encode_prep(const float* __restrict__ X, int64_t n, int d, const unsigned char
     nrm[row] = nr;
     // 0 for a zero row; also where the norm is not finite (its 1/norm is 0, and
     // a value that is not finite still gives NaN)
-    xs[row] = nr > 0.f && nr < INFINITY ? h_pow2(14 - max(h_exp(nr), -100)) : 0.f;
+    xs[row] = nr > 0.f && nr < INFINITY ? pow2f(14 - max(exp2_of(nr), -100)) : 0.f;
   }
 }
 
@@ -335,12 +320,12 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
         const uint64_t rh = r0 + (uint64_t)((uint32_t)s * (H_STAGE_BYTES >> 4)), rl = rh + (HR_BYTES >> 4);
         const uint32_t ah = tm + H_TM_A + (uint32_t)s * 32u, al = ah + 16u;
         const uint32_t more = kb != 0;
-        if (h_elect()) {
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < HK / 16; ++kk) {  // 16 values: 32 bytes of each R row, 8 TMEM columns of x
-            h_mma(dt, ah + kk * 8u, rh + kk * 2u, idesc, kk ? 1u : more);
-            h_mma(dt, ah + kk * 8u, rl + kk * 2u, idesc, 1u);
-            h_mma(dt, al + kk * 8u, rh + kk * 2u, idesc, 1u);
+            mma_f16_ta(dt, ah + kk * 8u, rh + kk * 2u, idesc, kk ? 1u : more);
+            mma_f16_ta(dt, ah + kk * 8u, rl + kk * 2u, idesc, 1u);
+            mma_f16_ta(dt, al + kk * 8u, rh + kk * 2u, idesc, 1u);
           }
           mma_commit(empty + s);
           if (kb == KB - 1) mma_commit(acc_full + set);
@@ -352,7 +337,7 @@ k_encode_h(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
         }
       }
     }
-    if (h_elect()) {
+    if (elect_one()) {
       mma_commit(fin);
       mbar_wait_drain(fin, 0);
     }

@@ -93,23 +93,6 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b,
       ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc<N>()), "r"(accumulate));
 }
 
-// Scores as unsigned integers of the same order (0 below every score's), for
-// the thresholds that the CTAs of a query share.
-__device__ __forceinline__ uint32_t order_bits(float s) {
-  const uint32_t b = __float_as_uint(s + 0.0f);
-  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
-}
-__device__ __forceinline__ float ordered(uint32_t o) {
-  return __uint_as_float(o & 0x80000000u ? o ^ 0x80000000u : ~o);
-}
-
-// A score and its row as one key, larger = better (score descending, id ascending).
-__device__ __forceinline__ uint64_t rank_key(float s, int id) {
-  return ((uint64_t)order_bits(s) << 32) | (uint32_t)~id;
-}
-__device__ __forceinline__ float key_score(uint64_t key) { return ordered((uint32_t)(key >> 32)); }
-__device__ __forceinline__ int key_id(uint64_t key) { return (int)~(uint32_t)key; }
-
 struct MmaSmem {
   uint32_t a, b, raw, tab, scale, dense, bars, lists, total;
 };

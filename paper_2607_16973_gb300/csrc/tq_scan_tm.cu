@@ -104,27 +104,11 @@ __host__ __device__ constexpr uint32_t tm_idesc(int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TM_M >> 4) << 24);
 }
 
-// D (f32, TMEM) += A (fp16, TMEM) x B (fp16, shared memory), M = 128, K = 16.
-__device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
-                                           uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
 // warp_wait whose usual case, a phase already complete, is one poll per lane.
 __device__ __forceinline__ bool all_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err,
                                          int where) {
   if (__all_sync(FULL, mbar_try_wait(bar, parity))) return true;
   return warp_wait(bar, parity, abort_flag, err, where);
-}
-
-// True in one lane of a converged warp.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n selp.u32 %0, 1, 0, e;\n}" : "=r"(p));
-  return p != 0;
 }
 
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
@@ -139,28 +123,8 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
       : "memory");
 }
 
-// 2^e as a float for -126 <= e <= 127.
-__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-// floor(log2 |x|) of a normal float.
-__device__ __forceinline__ int exp2_of(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFFu) - 127; }
-
 // Magnitudes the bounds are derived for (no product below over- or underflows).
 constexpr float TM_BIG = 0x1p60f, TM_SMALL = 0x1p-50f, TM_SMALL_SCALE = 0x1p-40f;
-
-// Scores and ids as one 64-bit key, larger = better (score descending, id
-// ascending): the score's bits made order-preserving above the id's complement.
-__device__ __forceinline__ uint32_t order_bits(float s) {  // 0 is below every score's
-  const uint32_t b = __float_as_uint(s + 0.0f);            // -0 ranks as +0
-  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
-}
-__device__ __forceinline__ float ordered(uint32_t o) {
-  return __uint_as_float(o & 0x80000000u ? o ^ 0x80000000u : ~o);
-}
-__device__ __forceinline__ uint64_t rank_key(float s, int id) {
-  return ((uint64_t)order_bits(s) << 32) | (uint32_t)~id;
-}
-__device__ __forceinline__ float key_score(uint64_t key) { return ordered((uint32_t)(key >> 32)); }
-__device__ __forceinline__ int key_id(uint64_t key) { return (int)~(uint32_t)key; }
 
 // Sorts one key per lane across the warp, best first.
 __device__ __noinline__ uint64_t warp_sort_keys(uint64_t x) {

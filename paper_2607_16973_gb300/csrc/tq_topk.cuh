@@ -516,6 +516,24 @@ __device__ __forceinline__ void cta_lists_out(float* ls, int* li, int nw, int k,
   }
 }
 
+// Scores as unsigned integers of the same order (0 below every score's), for
+// comparisons and thresholds (atomicMax).
+__device__ __forceinline__ uint32_t order_bits(float s) {
+  const uint32_t b = __float_as_uint(s + 0.0f);  // -0 ranks as +0
+  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float ordered(uint32_t o) {
+  return __uint_as_float(o & 0x80000000u ? o ^ 0x80000000u : ~o);
+}
+
+// A score and its row as one 64-bit key, larger = better (score descending, id
+// ascending): the score's ordered bits above the id's complement.
+__device__ __forceinline__ uint64_t rank_key(float s, int id) {
+  return ((uint64_t)order_bits(s) << 32) | (uint32_t)~id;
+}
+__device__ __forceinline__ float key_score(uint64_t key) { return ordered((uint32_t)(key >> 32)); }
+__device__ __forceinline__ int key_id(uint64_t key) { return (int)~(uint32_t)key; }
+
 // Launches `kernel`, with programmatic stream serialization when `pdl` (the
 // kernel then overlaps the tail of the one before it and waits for it with
 // griddep_wait before reading its results).
