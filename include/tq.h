@@ -200,7 +200,9 @@ tq_status tq_encode_ex(const float* X, int64_t n, int d, const float* R,
  *                calls may land boundary coordinates in different cells.
  *                (From d = 1024 on, 8-bit codes from 768; below, where such
  *                a coordinate weighs more in its row's scalar, it runs as
- *                tq_encode_planned and reads no workspace.)  The
+ *                tq_encode_planned and reads no workspace, so that scalars
+ *                written before and after agree to a few 10^-3; it is no less
+ *                accurate there.)  The
  *                workspace is free again when the call's work has finished.
  *                n up to 2^31 - 1024.
  * tq_encode_workspace_for  the same for one code width: 0 where
@@ -295,10 +297,14 @@ tq_status tq_search_workspace(int64_t nq, int64_t n, int d, int bits, int k,
  * Kernels (TQ_PATH_AUTO): batches of 16 or more queries over 2-, 4- or 8-bit
  * codes with d a multiple of 64 and k <= 64 run a tensor-core scan (fp16
  * products, float32 accumulation), filtered or not; the rest give the lookup
- * scan's results (float32 sums).  Unfiltered batches below 16 over 4-bit codes
- * (d a multiple of 256, k <= 32, enough rows) get them from a tensor-core scan
- * that bounds every score and float32 scores of the candidates the bounds
- * leave, bit for bit what the lookup scan returns.
+ * scan's results (float32 sums).  Batches below 16 over 4-bit codes (d a
+ * multiple of 256, k <= 32, enough rows; with a filter from two queries on) get
+ * them from a tensor-core scan that bounds every score and float32 scores of the
+ * candidates the bounds leave, bit for bit what the lookup scan returns.  Where
+ * the bounds do not settle a query (more than 32 near-equal vectors among the
+ * best in one CTA's rows, or anywhere a scalar that is not finite, or not zero
+ * but below 2^-40 in magnitude) the lookup scan runs for it after that, and the
+ * search takes as long as both.
  */
 tq_status tq_search(const float* Q, int64_t nq, int d, const float* R,
                     const float* centroids, int bits, const uint8_t* codes,

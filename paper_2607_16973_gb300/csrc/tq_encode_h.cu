@@ -19,9 +19,9 @@
 // kernel takes 7.1 ms and the norms' pass over X 0.95.  On top come X's way to
 // the SMs, once per chunk (about 2 ms), its split, which 8 warps just keep up
 // with (2.4 ms), and R's tiles (1 ms).  Measured at 999,000 x 1536, 4-bit: 20.1 ms
-// (TF32) -> 12.1 ms; 1,000 rows 375 -> 48 us; 40,003 x 768 at 8 bits 444 -> 184 us.
+// (TF32) -> 12.4 ms; 1,000 rows 375 -> 48 us; 40,003 x 768 at 8 bits 444 -> 181 us.
 // Two accumulators of 192 columns hide the read-out behind the next chunk; with
-// one of 256 it took 12.7 ms and 211 us.  Four converter groups (72 registers,
+// one of 256 it took 12.9 ms and 211 us.  Four converter groups (72 registers,
 // the epilogue spills) 14.0 ms; separate rings of 3 X and 5 R stages 13.7 ms.
 //
 // Work.  The items are (128-row panel, chunk of N output coordinates), panel by
@@ -594,14 +594,17 @@ int encode_h_chunk(int64_t n, int d) {
 
 }  // namespace
 
-// Where the fp16 encoder runs.  The two encoders decide about 2 in 100,000
+// Where the fp16 encoder runs: a matter of agreement with the TF32 encoder's
+// bytes, not of accuracy (against 64 bits it was the closer of the two wherever
+// measured).  The two decide about 2 in 100,000
 // coordinates, those next to a boundary, differently, and one such coordinate
 // moves its row's scalar by (c1^2 - c0^2) / 2, at the outermost boundary up to
 // 1.04 / d of its value for 2-bit, 1.4 / d for 3-bit, 1.6 / d for 4-bit codes,
 // times its calibration squared.  Over 999,000 rows the largest change of a
 // scalar measured was 4.1e-3 at d = 768, 3.0e-3 at 1024, 2.1e-3 at 1536.  The
-// outer boundaries of 8-bit codes are rarely reached (2.2e-3 at d = 768).  Below
-// these d the codes stay those of the TF32 encoder.
+// outer boundaries of 8-bit codes are rarely reached (2.2e-3 at d = 768, the one
+// d measured).  Below these d rows encoded now and rows encoded before
+// keep agreeing as closely as rows of the TF32 encoder do: its codes stay.
 bool encode_h_applies(int d, int bits) { return encode_tc_supported(d) && d >= (bits == 8 ? 768 : 1024); }
 
 size_t encode_h_workspace(int64_t n, int d) { return encode_h_applies(d, 8) ? h_ws(n, d).total : 256; }

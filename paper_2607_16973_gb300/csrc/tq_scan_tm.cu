@@ -349,10 +349,14 @@ k_scan_tm(const __grid_constant__ CUtensorMap codes_map, const float* __restrict
       if (fine) {
         // |fp16 score - lookup score| <= sum |q16 c16 - q c| (operand
         // rounding) + accumulation: the MMAs add d products to a float32 sum
-        // in d / 16 steps, each aligning 17 terms to the largest and cutting
-        // below its last bit: d * 2^-23 of sum |q c| covers that twice over,
-        // 2^-17 the lookup scan's own float32 rounding and the additions and
-        // products here.
+        // in d / 16 steps.  How a step rounds is not documented; if it aligns
+        // its 17 terms to the largest and cuts below its last bit, as was
+        // measured on earlier tensor cores (Fasi, Higham, Mikaitis and Pranesh,
+        // "Numerical behavior of NVIDIA tensor cores", 2021), d * 2^-23 of
+        // sum |q c| covers it twice over.  On GB300 the largest error of
+        // products far apart in magnitude, d = 256 and 2,048, was 0.025 of
+        // that (test_gpu_scan_tm.py).  2^-17 covers the lookup scan's own
+        // float32 rounding and the additions and products here.
         const float de = dq / qs, ce = cerr / cs;
         e = (l1 + de) * ce + de * cmax + l1 * cmax * ((float)d * 0x1p-23f + 0x1p-17f) + fabsf(bq) * 0x1p-20f;
         e *= 1.0001f;
