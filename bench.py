@@ -487,7 +487,7 @@ def run_ours(args, cfg, rank, world):
                 traffic = recorded_traffic(("paper_2607_16973_gb300/csrc/tq_fold.cu",
                                             "paper_2607_16973_gb300/csrc/tq_topk.cuh"), "k_scan_fold_250k_batch1.md",
                                            scale_to=n)
-            elif kern == "k_scan_stream" and bits == 4 and args.search_path == "auto":
+            elif kern == "k_scan_stream" and bits == 4 and args.search_path in ("auto", "lut"):
                 traffic = recorded_traffic(("paper_2607_16973_gb300/csrc/tq_scan.cu",
                                             "paper_2607_16973_gb300/csrc/tq_topk.cuh"), "k_scan_stream_250k_batch1.md",
                                            scale_to=n)
