@@ -519,32 +519,30 @@ int device_sm_count() {
 }
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel, device
-// and size: the call is not free, and the searches launch on every request.
+// and size: the call is not free, and the searches launch on every request.  It
+// only ever raises the attribute, and under the lock: two threads that raised it
+// for different sizes at once could leave the smaller one set.
 cudaError_t set_max_dynamic_smem(const void* func, int bytes) {
   struct Entry {
     const void* func;
     int dev, bytes;
   };
+  constexpr int kMaxSeen = 2048;
   static std::mutex mu;
-  static Entry seen[256];
+  static Entry seen[kMaxSeen];
   static int nseen = 0;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (int i = 0; i < nseen; ++i)
-      if (seen[i].func == func && seen[i].dev == dev && seen[i].bytes >= bytes) return cudaSuccess;
-  }
+  std::lock_guard<std::mutex> lock(mu);
+  Entry* entry = nullptr;
+  for (int i = 0; i < nseen && !entry; ++i)
+    if (seen[i].func == func && seen[i].dev == dev) entry = seen + i;
+  if (entry && entry->bytes >= bytes) return cudaSuccess;
   e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> lock(mu);
-  for (int i = 0; i < nseen; ++i)
-    if (seen[i].func == func && seen[i].dev == dev) {
-      if (bytes > seen[i].bytes) seen[i].bytes = bytes;
-      return cudaSuccess;
-    }
-  if (nseen < 256) seen[nseen++] = Entry{func, dev, bytes};
+  if (!entry && nseen < kMaxSeen) seen[nseen++] = Entry{func, dev, bytes};
+  else if (entry) entry->bytes = bytes;
   return cudaSuccess;
 }
 
