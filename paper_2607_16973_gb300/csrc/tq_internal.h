@@ -44,10 +44,9 @@ int& fail_allocs();
 inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
 inline int64_t row_bytes(int d, int bits) { return (int64_t)d * bits / 8; }
 // Tiles of `rows` rows that n rows take (n goes up to 2^31 - 2, where n + rows - 1
-// would wrap as an int).
-constexpr int row_tiles(int n, int rows) {
-  return (int)(((unsigned)n + (unsigned)rows - 1u) / (unsigned)rows);
-}
+// would wrap as an int).  In 64 bits: other forms that do not wrap (unsigned, or a
+// division and a remainder) gave the scans at d = 2048 more spilled registers.
+constexpr int row_tiles(int n, int rows) { return (int)(((int64_t)n + rows - 1) / rows); }
 static_assert(row_tiles(0x7FFFFFFE, 128) == 1 << 24 && row_tiles(0x7FFFFFFE, 4) == 1 << 29 &&
                   row_tiles(128, 128) == 1 && row_tiles(129, 128) == 2,
               "row tiles");
